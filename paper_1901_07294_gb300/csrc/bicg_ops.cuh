@@ -104,8 +104,8 @@ template <int P> struct OpBicgAlpha {
         v.load(j, b);
         T re = 0, im = 0;
         site_zdot(a, b, re, im);
-        acc[0] += (double)re;
-        acc[1] += (double)im;
+        acc[0] += to_real<double>(re);
+        acc[1] += to_real<double>(im);
     }
     __device__ __forceinline__ void finish(const double (&d)[2]) const
     {
@@ -137,7 +137,7 @@ template <int P> struct OpBicgS {
 #pragma unroll
         for (int k = 0; k < 24; ++k) n = fma(rv[k], rv[k], n);
         out.store(j, rv);
-        acc[0] += (double)n;
+        acc[0] += to_real<double>(n);
     }
     __device__ __forceinline__ void finish(const double (&d)[1]) const { s[BS_S2] = d[0]; }
 };
@@ -157,9 +157,9 @@ template <int P> struct OpBicgOmega {
         site_zdot(a, b, re, im);
 #pragma unroll
         for (int k = 0; k < 24; ++k) tt = fma(a[k], a[k], tt);
-        acc[0] += (double)re;
-        acc[1] += (double)im;
-        acc[2] += (double)tt;
+        acc[0] += to_real<double>(re);
+        acc[1] += to_real<double>(im);
+        acc[2] += to_real<double>(tt);
     }
     __device__ __forceinline__ void finish(const double (&d)[3]) const
     {
@@ -201,9 +201,9 @@ template <int PX, int P> struct OpBicgUpdate {
         for (int k = 0; k < 24; ++k) n = fma(svv[k], svv[k], n);
         site_zdot(hv, svv, re, im);
         r.store(j, svv);
-        acc[0] += (double)n;
-        acc[1] += (double)re;
-        acc[2] += (double)im;
+        acc[0] += to_real<double>(n);
+        acc[1] += to_real<double>(re);
+        acc[2] += to_real<double>(im);
     }
     __device__ __forceinline__ void finish(const double (&d)[3]) const
     {
@@ -234,8 +234,8 @@ template <int P> struct OpBicgRho {
         r.load(j, b);
         T re = 0, im = 0;
         site_zdot(a, b, re, im);
-        acc[0] += (double)re;
-        acc[1] += (double)im;
+        acc[0] += to_real<double>(re);
+        acc[1] += to_real<double>(im);
     }
     __device__ __forceinline__ void finish(const double (&d)[2]) const
     {
@@ -266,7 +266,7 @@ template <int P> struct OpBicgRestart {
         T n = 0;
 #pragma unroll
         for (int k = 0; k < 24; ++k) n = fma(rv[k], rv[k], n);
-        acc[0] += (double)n;
+        acc[0] += to_real<double>(n);
     }
     __device__ __forceinline__ void finish(const double (&d)[1]) const
     {

@@ -47,14 +47,19 @@ template <typename Op> inline int blas_resident_blocks()
 // thread up to the blocks that fit on the device at once, longer fields
 // looping within it (a partial second wave, as with a fixed 8 blocks per SM
 // for a kernel that fits 6, leaves the last blocks' partial sums, and so the
-// final sum, waiting on its stragglers).  Operations without a reduction keep
+// final sum, waiting on its stragglers), and with at most 4 blocks per SM: every
+// block costs a block sum on the FP64 pipe and a partial that the last block
+// has to add (24^3 x 48 half fields, FP16: inner product 9.1 us with all the
+// blocks that fit, 8.4 with 4 or 3 per SM, 9.0 with 2, 11.3 with 1; FP64 norm
+// on 32^4 31.9, 27.5, 26.7, 32.4).  Operations without a reduction keep
 // blas_grid.  Fixed by the field size, the SM count and the kernel, so the
 // reduction order is too.
 template <typename Op> inline int blas_grid_for(const wd_ctx *ctx, int nsite)
 {
     if constexpr (Op::NR == 0) return blas_grid(ctx, nsite);
     const int want = (nsite + BLAS_THREADS - 1) / BLAS_THREADS;
-    int cap = blas_resident_blocks<Op>() * (ctx->num_sms > 0 ? ctx->num_sms : 132);
+    const int fit = blas_resident_blocks<Op>();
+    int cap = (fit < 4 ? fit : 4) * (ctx->num_sms > 0 ? ctx->num_sms : 132);
     if (cap > MAX_RED_BLOCKS) cap = MAX_RED_BLOCKS;
     return want < cap ? (want > 0 ? want : 1) : cap;
 }
