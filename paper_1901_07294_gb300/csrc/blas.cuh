@@ -260,64 +260,63 @@ template <int P, int PY = P> struct OpXmyNorm {
     __device__ __forceinline__ void finish(const double (&s)[1]) const { out[0] = s[0]; }
 };
 
-// ---- CG steps whose scalars live in device memory (replayable in a graph) ----
-// Scalar slots: s[0] = |r|^2 now, s[1] = pAp, s[2] = alpha, s[4] = |r|^2 of
-// the previous step, s[5] = beta for the next direction update, s[6] =
-// breakdown flag.
-
-// pAp = Re<p, Ap>;  alpha = s[0] / pAp  (alpha = 0 and the flag set on breakdown)
-template <int P> struct OpDotAlphaDev {
-    static constexpr int NR = 1;
-    FieldRef<P> p, q;
-    double *s;
-    __device__ __forceinline__ void site(int j, double (&acc)[1]) const
-    {
-        typename Prec<P>::real u[24], w[24];
-        p.load(j, u);
-        q.load(j, w);
-        typename Prec<P>::real t = 0;
-#pragma unroll
-        for (int k = 0; k < 24; ++k) t = fma(u[k], w[k], t);
-        acc[0] += to_real<double>(t);
-    }
-    __device__ __forceinline__ void finish(const double (&r)[1]) const
-    {
-        s[1] = r[0];
-        const bool ok = r[0] > 0.0 && r[0] < 1e300;
-        s[2] = ok ? s[0] / r[0] : 0.0;
-        if (!ok) s[6] = 1.0;
-    }
-};
-
-// r -= alpha Ap; x += alpha p (alpha = s[2]); then s[4] = s[0], s[0] = |r|^2.
-template <int PX, int PR> struct OpCgUpdateDev {
-    static constexpr int NR = 1;
-    OpCgUpdate<PX, PR> u;
-    double *s;
-    __device__ __forceinline__ void site(int j, double (&acc)[1]) const { u.site(j, acc); }
-    __device__ __forceinline__ void finish(const double (&r)[1]) const
-    {
-        s[4] = s[0];
-        s[0] = r[0];
-    }
-};
-
-// p = r + beta p with beta = s[5] (= s[0] / s[4], set once per iteration by the
-// solve's control step, or by the host after a reliable update)
-template <int P> struct OpXpayDev {
+// ---- vector updates of the mixed-precision CG iteration ----------------------
+// x += alpha p, then p = r + beta p: the vector updates left to a kernel of their
+// own when the hops carry the rest (dslash_cg.cuh).  alpha is read from device
+// memory, beta too unless beta_dev is NULL.  x may have another precision.
+template <int PX, int P> struct OpXp {
     static constexpr int NR = 0;
+    FieldRef<PX> x;
     FieldRef<P> r, p;
-    const double *s;
+    const double *alpha, *beta_dev;
+    double beta;
     __device__ __forceinline__ void site(int j, double (&)[1]) const
     {
         using T = typename Prec<P>::real;
-        const T beta = (T)s[5];
+        using TX = typename Prec<PX>::real;
+        const TX al = (TX)*alpha;
+        const T be = (T)(beta_dev ? *beta_dev : beta);
         T rv[24], pv[24];
-        r.load(j, rv);
+        TX xv[24];
         p.load(j, pv);
+        x.load(j, xv);
+        r.load(j, rv);
 #pragma unroll
-        for (int k = 0; k < 24; ++k) pv[k] = fma(beta, pv[k], rv[k]);
+        for (int k = 0; k < 24; ++k) {
+            xv[k] = fma(al, to_real<TX>(pv[k]), xv[k]);
+            pv[k] = fma(be, pv[k], rv[k]);
+        }
+        x.store(j, xv);
         p.store(j, pv);
+    }
+    __device__ __forceinline__ void finish(const double (&)[1]) const {}
+};
+
+// x += x_lo + alpha p for the FP64 solution x, and x_lo = 0: the start of a
+// reliable update, with the step of the last iteration (not yet in x_lo)
+template <int PX, int P> struct OpFlushX {
+    static constexpr int NR = 0;
+    FieldRef<PREC_F64> x;
+    FieldRef<PX> xlo;
+    FieldRef<P> p;
+    const double *alpha;
+    __device__ __forceinline__ void site(int j, double (&)[1]) const
+    {
+        using TX = typename Prec<PX>::real;
+        const TX al = (TX)*alpha;
+        double xv[24];
+        TX lo[24];
+        typename Prec<P>::real pv[24];
+        xlo.load(j, lo);
+        p.load(j, pv);
+        x.load(j, xv);
+#pragma unroll
+        for (int k = 0; k < 24; ++k) {
+            xv[k] += to_real<double>(fma(al, to_real<TX>(pv[k]), lo[k]));
+            lo[k] = TX(0);
+        }
+        x.store(j, xv);
+        xlo.store(j, lo);
     }
     __device__ __forceinline__ void finish(const double (&)[1]) const {}
 };

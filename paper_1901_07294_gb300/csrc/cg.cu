@@ -59,6 +59,20 @@ int read_scalars(wd_ctx *ctx, int first, int n, cudaStream_t s)
     return WD_OK;
 }
 
+// s[0] = s[3] = the sum of the n site sums.
+__global__ void __launch_bounds__(256) site_norm_kernel(const float *site, int n, double *s, RedScratch red)
+{
+    grid_dependency_enter();
+    site_sum(site, n, blockIdx.x, gridDim.x, red, [&](double v) { s[0] = s[3] = v; });
+}
+
+int site_norm(wd_ctx *ctx, const float *site, int n, double *s, cudaStream_t stream)
+{
+    const cudaError_t e = wd_launch(site_norm_kernel, dim3(cg_parts(n, 256)), dim3(256), 0, stream, site, n, s,
+                                    RedScratch{ctx->d_partials, ctx->d_ticket});
+    return e == cudaSuccess ? WD_OK : set_error(WD_ECUDA, "BLAS kernel launch failed: %s", cudaGetErrorString(e));
+}
+
 template <int PS, int PX>
 int cg_run(wd_ctx *ctx, const wd_gauge *g, double mass, char *x, const char *b, double tol, const wd_cg_opts &o,
            wd_cg_stats &st, cudaStream_t s)
@@ -110,9 +124,15 @@ int cg_run(wd_ctx *ctx, const wd_gauge *g, double mass, char *x, const char *b, 
     int status = WD_OK;
     int it = 0, it_update = 0;
     while (it < o.maxiter) {
-        WD_TRY(apply_mdagm(g, PS, o.inner_recon, mass, ps, aps, tso, tse, s));
-        WD_TRY(run_blas(ctx, OpDotReAlpha<PS>{FS(ps), FS(aps), r2, d + 1}, vh, s));   // d1 = pAp, d2 = alpha
-        WD_TRY(run_blas(ctx, OpCgUpdate<PX, PS>{FX(xs), FS(rs), FS(ps), FS(aps), d + 2, d + 3}, vh, s));
+        if constexpr (PS == PREC_F64) {
+            WD_TRY(apply_mdagm(g, PS, o.inner_recon, mass, ps, aps, tso, tse, s));
+            WD_TRY(run_blas(ctx, OpDotReAlpha<PS>{FS(ps), FS(aps), r2, d + 1}, vh, s));   // d1 = pAp, d2 = alpha
+            WD_TRY(run_blas(ctx, OpCgUpdate<PX, PS>{FX(xs), FS(rs), FS(ps), FS(aps), d + 2, d + 3}, vh, s));
+        } else {   // d1 = pAp, d2 = alpha, r updated, d3 = |r|^2; x takes its step with the next p
+            WD_TRY(cg_iteration_hops(g, PS, o.inner_recon, mass,
+                                     CgFields{ps, rs, tso, tse, (float *)aps, d, ctx->d_partials, ctx->d_ticket}, s));
+            WD_TRY(site_norm(ctx, (const float *)aps, vh, d, s));
+        }
         WD_TRY(read_scalars(ctx, 1, 3, s));
         ++it;
         const double pap = h[1];
@@ -132,8 +152,12 @@ int cg_run(wd_ctx *ctx, const wd_gauge *g, double mass, char *x, const char *b, 
         else update = r2_new <= std::fmax(stop2, delta * delta * r2_restart);
         if (update) {
             // x += x_lo (FP64), then the true residual with the FP64 operator
-            WD_TRY(run_blas(ctx, OpAxpby<PX, PREC_F64>{FX(xs), F64(x), 1.0, 1.0}, vh, s));
-            WD_CUDA_TRY(cudaMemsetAsync(xs, 0, hx, s));
+            if constexpr (PS == PREC_F64) {
+                WD_TRY(run_blas(ctx, OpAxpby<PX, PREC_F64>{FX(xs), F64(x), 1.0, 1.0}, vh, s));
+                WD_CUDA_TRY(cudaMemsetAsync(xs, 0, hx, s));
+            } else {
+                WD_TRY(run_blas(ctx, OpFlushX<PX, PS>{F64(x), FX(xs), FS(ps), d + 2}, vh, s));
+            }
             // an update that the iterated residual's convergence triggered is a
             // convergence check: FP64 directly, as are all updates after a failed check
             const bool check = r2_new <= stop2;
@@ -161,6 +185,8 @@ int cg_run(wd_ctx *ctx, const wd_gauge *g, double mass, char *x, const char *b, 
                 break;
             }
             WD_TRY(run_blas(ctx, OpConvert<PS, PREC_F64>{FS(rs), F64(r)}, vh, s));
+            if (PS != PREC_F64)   // |r|^2 of the next step length
+                WD_CUDA_TRY(cudaMemcpyAsync(d, d + 4, sizeof(double), cudaMemcpyDeviceToDevice, s));
             r2_new = r2_true;
             maxr = std::sqrt(r2_true);
             if (!reliable) {   // iterative refinement: restart the inner CG on the new residual
@@ -171,7 +197,10 @@ int cg_run(wd_ctx *ctx, const wd_gauge *g, double mass, char *x, const char *b, 
             }
         }
         const double beta = r2_new / r2;
-        WD_TRY(run_blas(ctx, OpAxpby<PS, PS>{FS(rs), FS(ps), 1.0, beta}, vh, s));   // p = r + beta p
+        if (PS == PREC_F64 || update)   // p = r + beta p; with x += alpha p unless an update has taken that step
+            WD_TRY(run_blas(ctx, OpAxpby<PS, PS>{FS(rs), FS(ps), 1.0, beta}, vh, s));
+        else
+            WD_TRY(run_blas(ctx, OpXp<PX, PS>{FX(xs), FS(rs), FS(ps), d + 2, nullptr, beta}, vh, s));
         r2 = r2_new;
     }
     if (!converged && status == WD_OK) {

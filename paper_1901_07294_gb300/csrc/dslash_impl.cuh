@@ -260,14 +260,13 @@ __device__ __forceinline__ void hop_dir(const char *in, const char *lblk, int vh
     accumulate<MU, S, FIRST>(acc, w0, w1);
 }
 
-// 16-bit storage: out = a x + acc at site i, with acc the sum already
+// 16-bit storage: o = a x + acc at site i, with acc the sum already
 // weighted by the hop coefficient (hop_dir's wt); x is read as stored and its
 // per-site scale folded into a.
 template <int P, bool HAS_X>
-__device__ __forceinline__ void store_weighted(const char *x, char *out, int vh, int i, float a,
-                                               const cpx<float> (&acc)[4][3])
+__device__ __forceinline__ void value_weighted(const char *x, int vh, int i, float a, const cpx<float> (&acc)[4][3],
+                                               float (&o)[24])
 {
-    float o[24];
     if constexpr (HAS_X) {
         unsigned u[12];
         const float ax = a * Spinor<P>::load_words(x, vh, i, u);
@@ -287,8 +286,66 @@ __device__ __forceinline__ void store_weighted(const char *x, char *out, int vh,
                 o[6 * s + 2 * c + 1] = acc[s][c].im;
             }
     }
+}
+
+template <int P, bool HAS_X>
+__device__ __forceinline__ void store_weighted(const char *x, char *out, int vh, int i, float a,
+                                               const cpx<float> (&acc)[4][3])
+{
+    float o[24];
+    value_weighted<P, HAS_X>(x, vh, i, a, acc, o);
     Spinor<P>::store(out, vh, i, o);
 }
+
+// o = a x + b acc at site i of parity p, field at byte offset roff (16-bit
+// storage: acc already carries b).
+template <int P, bool HAS_X>
+__device__ __forceinline__ void hop_value(const HopArgs &A, int p, int i, size_t roff,
+                                          const cpx<typename Prec<P>::real> (&acc)[4][3],
+                                          typename Prec<P>::real (&o)[24])
+{
+    using T = typename Prec<P>::real;
+    const T a = (T)A.a, b = (T)A.b;
+    if constexpr (Prec<P>::scaled) {
+        value_weighted<P, HAS_X>(HAS_X ? (p ? A.x[1] : A.x[0]) + roff : nullptr, A.vh, i, (float)A.a, acc, o);
+    } else if constexpr (HAS_X) {
+        Spinor<P>::load((p ? A.x[1] : A.x[0]) + roff, A.vh, i, o);
+#pragma unroll
+        for (int s = 0; s < 4; ++s)
+#pragma unroll
+            for (int c = 0; c < 3; ++c) {
+                o[6 * s + 2 * c] = a * o[6 * s + 2 * c] + b * acc[s][c].re;
+                o[6 * s + 2 * c + 1] = a * o[6 * s + 2 * c + 1] + b * acc[s][c].im;
+            }
+    } else if (A.b == 1.0) {   // the bare hopping term: no scaling
+#pragma unroll
+        for (int s = 0; s < 4; ++s)
+#pragma unroll
+            for (int c = 0; c < 3; ++c) {
+                o[6 * s + 2 * c] = acc[s][c].re;
+                o[6 * s + 2 * c + 1] = acc[s][c].im;
+            }
+    } else {
+#pragma unroll
+        for (int s = 0; s < 4; ++s)
+#pragma unroll
+            for (int c = 0; c < 3; ++c) {
+                o[6 * s + 2 * c] = b * acc[s][c].re;
+                o[6 * s + 2 * c + 1] = b * acc[s][c].im;
+            }
+    }
+}
+
+// What a hop does with its site's sum: the operator stores out = a x + b acc.
+template <int P, bool HAS_X> struct HopStore {
+    __device__ __forceinline__ void operator()(const HopArgs &A, int p, int i, size_t roff,
+                                               const cpx<typename Prec<P>::real> (&acc)[4][3]) const
+    {
+        typename Prec<P>::real o[24];
+        hop_value<P, HAS_X>(A, p, i, roff, acc, o);
+        Spinor<P>::store((p ? A.out[1] : A.out[0]) + roff, A.vh, i, o);
+    }
+};
 
 // PF selects the memory schedule (chosen per problem by the autotuner):
 //   0: directions in the order x+, x-, y+, y-, ..., no prefetch;
@@ -301,8 +358,10 @@ __device__ __forceinline__ void store_weighted(const char *x, char *out, int vh,
 // at byte offset roff.  Shared by hop_kernel and the persistent solver.
 // TOPEN: the t boundary is open (a sub-domain of a decomposed lattice): the
 // hops across it are skipped; their halo terms are added separately.
-template <int P, int RECON, bool DAG, bool HAS_X, int PF, bool TOPEN = false, bool LNA = false>
-__device__ __forceinline__ void hop_site(const HopArgs &A, const int p, const int i, const size_t roff)
+template <int P, int RECON, bool DAG, bool HAS_X, int PF, bool TOPEN = false, bool LNA = false,
+          typename Epi = HopStore<P, HAS_X>>
+__device__ __forceinline__ void hop_site(const HopArgs &A, const int p, const int i, const size_t roff,
+                                         const Epi &epi = Epi())
 {
     using T = typename Prec<P>::real;
     const int vh = A.vh;
@@ -373,6 +432,13 @@ __device__ __forceinline__ void hop_site(const HopArgs &A, const int p, const in
         if (dtf) hop_dir<P, RECON, 3, SF, true, LNA>(in, gf + 3 * lb, vh, tf, i, ntf, acc, wt);
     }
 
+    if constexpr (!std::is_same_v<Epi, HopStore<P, HAS_X>>) {
+        epi(A, p, i, roff, acc);
+        return;
+    }
+    // HopStore, spelled out: through hop_value the compiler orders the FP32
+    // kernel's loads differently and the full operator on 32^4 takes 93 instead
+    // of 88 us
     const T a = (T)A.a, b = (T)A.b;
     T o[24];
     if constexpr (Prec<P>::scaled) {   // acc already carries b

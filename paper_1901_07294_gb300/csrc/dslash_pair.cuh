@@ -147,8 +147,9 @@ __device__ __forceinline__ void sp_dir(const char *in, const char *lblk, int vh,
 // of hop_site (backward directions first, forward links and t-forward
 // neighbour prefetched into L2); PF 0: schedule 0 (natural order, no
 // prefetch).  LNA: links loaded without L1 allocation.
-template <int P, int RECON, bool DAG, bool HAS_X, int PF, bool LNA>
-__device__ __forceinline__ void sp_site(const HopArgs &A, const int p, const int i, const size_t roff)
+template <int P, int RECON, bool DAG, bool HAS_X, int PF, bool LNA, typename Epi = HopStore<P, HAS_X>>
+__device__ __forceinline__ void sp_site(const HopArgs &A, const int p, const int i, const size_t roff,
+                                        const Epi &epi = Epi())
 {
     const int vh = A.vh;
     const char *in = (p ? A.in[1] : A.in[0]) + roff;
@@ -217,8 +218,7 @@ __device__ __forceinline__ void sp_site(const HopArgs &A, const int p, const int
         v[2][c] = {acc.l23[c].re.x + acc.l32[c].re.y, acc.l23[c].im.x + acc.l32[c].im.y};
         v[3][c] = {acc.l23[c].re.y + acc.l32[c].re.x, acc.l23[c].im.y + acc.l32[c].im.x};
     }
-    store_weighted<P, HAS_X>(HAS_X ? (p ? A.x[1] : A.x[0]) + roff : nullptr, (p ? A.out[1] : A.out[0]) + roff, vh, i,
-                             (float)A.a, v);
+    epi(A, p, i, roff, v);
 }
 
 template <int P, int RECON, bool DAG, bool HAS_X, int PF, bool LNA>

@@ -5,8 +5,10 @@
 // inner link format iterate together: each of the four even-odd hops of an
 // iteration is one launch of a shared-link kernel over all active members
 // (the links of 32 sites staged once in shared memory and applied to every
-// member's field, as in the multi right-hand-side kernel), and each BLAS step
-// is one launch with a row of blocks per member.  A member keeps its own
+// member's field, as in the multi right-hand-side kernel) that carries the
+// members' step lengths and residual updates as in dslash_cg.cuh, and the
+// update of x and p and the sum of |r|^2 are one launch each with rows of
+// blocks for the members.  A member keeps its own
 // workspace (a GSolve's fields, scalars and reduction scratch); the group only
 // holds a device table of the members' pointers and masses.  Per member the
 // arithmetic is the same whatever the other members are: its hops read only
@@ -35,10 +37,11 @@ template <int P> __host__ __device__ constexpr size_t half_bytes_p(int vh) { ret
 constexpr int GG_MAX = 32;          // members of one group at most
 constexpr int GG_LAUNCH_CAP = 16;   // iterations at most per group launch
 
-enum { GF_RS = 0, GF_PS = 1, GF_APS = 2, GF_TSO = 3, GF_TSE = 4 };
+enum { GF_RS = 0, GF_PS = 1, GF_TSO = 2, GF_TSE = 3 };
 
 struct GMember {
-    char *f[5];        // rs, ps, aps, tso, tse: inner-precision even/odd half fields
+    char *f[4];        // rs, ps, tso, tse: inner-precision even/odd half fields
+    float *site;       // per-site sums
     char *xs;          // FP32 solution increment since the last reliable update
     double *scal;      // the member's CG scalars (see gsolve.cuh)
     RedScratch red;    // its reduction scratch
@@ -48,16 +51,26 @@ struct GMember {
 struct GTable {
     int n;                 // members in this launch
     int launch_iters;      // iterations run in this launch (reset by the host)
+    unsigned done;         // members whose iteration has been summed up, and whether
+    unsigned stop;         // any of them must leave the loop (both 0 between iterations)
     int idx[GG_MAX];       // their member slots
     GMember m[GG_MAX];     // by slot
 };
 
 // ---- shared-link hop over the active members --------------------------------
-// Even-odd hop of output parity A.parity0 for every active member: out = f[fo],
-// in = f[fi], and with HAS_X the Mhat epilogue out = ma x + mc acc (x = f[fx]);
-// without, out = acc.  blockDim = (32, RY): warp y takes members y, y + RY, ...
-template <int P, int RECON, bool DAG, bool HAS_X>
-__global__ void __launch_bounds__(128, P == PREC_F64 ? 1 : 6)
+// Even-odd hop of output parity A.parity0 for every active member, with the
+// vector work of dslash_cg.cuh; blockDim = (32, RY): warp y takes members y,
+// y + RY, ...
+//   STEP 0         out = f[fo] = acc, in = f[fi];
+//   CG_NORM        out = f[fo] = ma x + mc acc (x = f[fx]), each site's |out|^2;
+//   CG_ALPHA       as 0, and the first blocks add the members' site sums (the
+//                  parts of all members shared out evenly) and set their alphas;
+//   CG_RESID       r = f[GF_RS] -= alpha (ma x + mc acc), each site's |r|^2.
+constexpr int GG_SUM_THREADS = 128;   // threads of a hop block
+constexpr int GG_SUM_BLOCKS = 64;   // blocks of a CG_ALPHA launch that add site sums
+
+template <int P, int RECON, bool DAG, int STEP>
+__global__ void __launch_bounds__(128, 6)
     hop_group_kernel(const HopArgs A, const GTable *__restrict__ T, const int fi, const int fx, const int fo)
 {
     grid_dependency_enter();
@@ -70,7 +83,22 @@ __global__ void __launch_bounds__(128, P == PREC_F64 ? 1 : 6)
     const int p = A.parity0;
     const int vh = A.vh;
     const int s = threadIdx.x;
-    const int i0 = blockIdx.x * 32 + s;
+    constexpr bool HAS_X = STEP == CG_NORM || STEP == CG_RESID;
+    int blk = blockIdx.x;
+    if constexpr (STEP == CG_ALPHA) {
+        if (blk < GG_SUM_BLOCKS) {
+            const int parts = cg_parts(vh, GG_SUM_THREADS);
+            for (int j = blk; j < n * parts; j += GG_SUM_BLOCKS) {
+                const GMember &m = T->m[T->idx[j / parts]];
+                site_sum(m.site, vh, j % parts, parts, m.red, [&](double v) { cg_set_alpha(m.scal, v); });
+                __syncthreads();   // the next sum reuses site_sum's shared memory
+            }
+            return;
+        }
+        blk -= GG_SUM_BLOCKS;
+    }
+    if constexpr (HAS_X) blk = gridDim.x - 1 - blk;   // every second hop backwards, as in hop_cg_kernel
+    const int i0 = blk * 32 + s;
     const bool active = i0 < vh;
     const int i = active ? i0 : -1;
     const char *gf = p ? A.gauge[1] : A.gauge[0];
@@ -122,12 +150,10 @@ __global__ void __launch_bounds__(128, P == PREC_F64 ? 1 : 6)
         hop_dir_smem<P, 1, SF, true>(in, vh, nb[32], &lk[1][0][s], false, acc, wt);
         hop_dir_smem<P, 2, SF, true>(in, vh, nb[64], &lk[2][0][s], false, acc, wt);
         hop_dir_smem<P, 3, SF, true>(in, vh, nb[96], &lk[3][0][s], A.tneg && nb[96] < i, acc, wt);
-        if constexpr (Prec<P>::scaled) {
-            store_weighted<P, HAS_X>(HAS_X ? m.f[fx] : nullptr, m.f[fo], vh, i, (float)m.ma, acc);
-            continue;
-        }
         T_ o[24];
-        if constexpr (HAS_X) {
+        if constexpr (Prec<P>::scaled) {
+            value_weighted<P, HAS_X>(HAS_X ? m.f[fx] : nullptr, vh, i, (float)m.ma, acc, o);
+        } else if constexpr (HAS_X) {
             const T_ a = (T_)m.ma, b = (T_)m.mc;
             Spinor<P>::load(m.f[fx], vh, i, o);
 #pragma unroll
@@ -146,7 +172,9 @@ __global__ void __launch_bounds__(128, P == PREC_F64 ? 1 : 6)
                     o[6 * sp + 2 * c + 1] = acc[sp][c].im;
                 }
         }
-        Spinor<P>::store(m.f[fo], vh, i, o);
+        if constexpr (STEP == CG_NORM) m.site[i] = site_norm2(o);
+        if constexpr (STEP == CG_RESID) m.site[i] = cg_residual<P>(m.f[GF_RS], vh, i, (float)m.scal[2], o);
+        else Spinor<P>::store(m.f[fo], vh, i, o);
     }
 }
 
@@ -156,66 +184,48 @@ __global__ void __launch_bounds__(128, P == PREC_F64 ? 1 : 6)
 // group's size, and a small group launches no rows of blocks with nothing to do.
 constexpr int GG_BLAS_ROWS = 8;
 
-template <int PS> __global__ void __launch_bounds__(BLAS_THREADS) gg_xpay_kernel(const GTable *__restrict__ T, int vh)
-{
-    grid_dependency_enter();
-    const size_t hs = half_bytes_p<PS>(vh);
-    for (int t = blockIdx.y; t < T->n; t += gridDim.y) {
-        const GMember &m = T->m[T->idx[t]];
-        blas_body(OpXpayDev<PS>{FieldRef<PS>{m.f[GF_RS], hs, vh}, FieldRef<PS>{m.f[GF_PS], hs, vh}, m.scal}, vh, m.red);
-        __syncthreads();   // the next member reuses blas_body's shared memory
-    }
-}
-
-template <int PS> __global__ void __launch_bounds__(BLAS_THREADS) gg_dot_kernel(const GTable *__restrict__ T, int vh)
-{
-    grid_dependency_enter();
-    const size_t hs = half_bytes_p<PS>(vh);
-    for (int t = blockIdx.y; t < T->n; t += gridDim.y) {
-        const GMember &m = T->m[T->idx[t]];
-        blas_body(OpDotAlphaDev<PS>{FieldRef<PS>{m.f[GF_PS], hs, vh}, FieldRef<PS>{m.f[GF_APS], hs, vh}, m.scal}, vh,
-                  m.red);
-        __syncthreads();   // the next member reuses blas_body's shared memory
-    }
-}
-
-template <int PS> __global__ void __launch_bounds__(BLAS_THREADS) gg_update_kernel(const GTable *__restrict__ T, int vh)
+template <int PS> __global__ void __launch_bounds__(BLAS_THREADS) gg_xp_kernel(const GTable *__restrict__ T, int vh)
 {
     grid_dependency_enter();
     const size_t hs = half_bytes_p<PS>(vh), h32 = half_bytes_p<PREC_F32>(vh);
     for (int t = blockIdx.y; t < T->n; t += gridDim.y) {
         const GMember &m = T->m[T->idx[t]];
-        OpCgUpdateDev<PREC_F32, PS> up{OpCgUpdate<PREC_F32, PS>{FieldRef<PREC_F32>{m.xs, h32, vh},
-                                                               FieldRef<PS>{m.f[GF_RS], hs, vh},
-                                                               FieldRef<PS>{m.f[GF_PS], hs, vh},
-                                                               FieldRef<PS>{m.f[GF_APS], hs, vh}, m.scal + 2, nullptr},
-                                       m.scal};
-        blas_body(up, vh, m.red);
-        __syncthreads();   // the next member reuses blas_body's shared memory
+        blas_body(OpXp<PREC_F32, PS>{FieldRef<PREC_F32>{m.xs, h32, vh}, FieldRef<PS>{m.f[GF_RS], hs, vh},
+                                     FieldRef<PS>{m.f[GF_PS], hs, vh}, m.scal + 2, m.scal + 5, 0.0}, vh, m.red);
     }
 }
 
-// The loop condition: each active member's bookkeeping as in gs_control_kernel
-// (without the per-launch count, kept once for the group); the loop stops when
-// any member stops or the group has run GG_LAUNCH_CAP iterations.  The
-// members' scalars are copied to `hs` (GS_NSCAL per active position) for the
-// host to read after the launch.
-__global__ void gg_control_kernel(GTable *T, double *hs, cudaGraphConditionalHandle cond)
+// The end of an iteration: each active member's |r|^2 from its site sums and its
+// bookkeeping as in gs_control_kernel (without the per-launch count, kept once
+// for the group); the loop stops when any member stops or the group has run
+// GG_LAUNCH_CAP iterations.  The members' scalars are copied to `hs` (GS_NSCAL
+// per active position) for the host to read after the launch.
+__global__ void __launch_bounds__(BLAS_THREADS)
+    gg_control_kernel(GTable *T, double *hs, int vh, cudaGraphConditionalHandle cond)
 {
     grid_dependency_enter();
-    const int t = threadIdx.x;
     const int n = T->n;
-    bool stop = false;
-    if (t < n) {
-        double *s = T->m[T->idx[t]].scal;
-        stop = gs_member_step(s);
-        for (int k = 0; k < GS_NSCAL; ++k) hs[t * GS_NSCAL + k] = s[k];
+    if (n == 0) {
+        if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) cudaGraphSetConditional(cond, 0u);
+        return;
     }
-    stop = __syncthreads_or(stop);
-    if (t == 0) {
-        const int li = T->launch_iters + 1;
-        T->launch_iters = li;
-        cudaGraphSetConditional(cond, (stop || n == 0 || li >= GG_LAUNCH_CAP) ? 0u : 1u);
+    for (int t = blockIdx.y; t < n; t += gridDim.y) {
+        const GMember &m = T->m[T->idx[t]];
+        site_sum(m.site, vh, blockIdx.x, gridDim.x, m.red, [&](double v) {
+            double *s = m.scal;
+            s[4] = s[0];
+            s[0] = v;
+            if (gs_member_step(s)) atomicOr(&T->stop, 1u);
+            for (int k = 0; k < GS_NSCAL; ++k) hs[t * GS_NSCAL + k] = s[k];
+            if (ticket_take(&T->done) == (unsigned)n - 1u) {   // the last member
+                const int li = T->launch_iters + 1;
+                T->launch_iters = li;
+                const unsigned stop = atomicExch(&T->stop, 0u);
+                T->done = 0u;
+                cudaGraphSetConditional(cond, (stop || li >= GG_LAUNCH_CAP) ? 0u : 1u);
+            }
+        });
+        __syncthreads();   // the next member reuses site_sum's shared memory
     }
 }
 
@@ -261,21 +271,21 @@ template <int PS> int build(const wd_ctx *ctx, GGroup &g)
     HopArgs Ao = A, Ae = A;
     Ao.parity0 = WD_ODD;
     Ae.parity0 = WD_EVEN;
-    wd_launch(gg_xpay_kernel<PS>, bgrid, bblk, 0, g.s, T, vh);
+    const dim3 hgrid_sum(hgrid.x + GG_SUM_BLOCKS);
+    wd_launch(gg_xp_kernel<PS>, bgrid, bblk, 0, g.s, T, vh);
     if (g.recon == 12) {
-        wd_launch(hop_group_kernel<PS, 12, false, false>, hgrid, hblk, 0, g.s, Ao, T, (int)GF_PS, 0, (int)GF_TSO);
-        wd_launch(hop_group_kernel<PS, 12, false, true>, hgrid, hblk, 0, g.s, Ae, T, (int)GF_TSO, (int)GF_PS, (int)GF_TSE);
-        wd_launch(hop_group_kernel<PS, 12, true, false>, hgrid, hblk, 0, g.s, Ao, T, (int)GF_TSE, 0, (int)GF_TSO);
-        wd_launch(hop_group_kernel<PS, 12, true, true>, hgrid, hblk, 0, g.s, Ae, T, (int)GF_TSO, (int)GF_TSE, (int)GF_APS);
+        wd_launch(hop_group_kernel<PS, 12, false, 0>, hgrid, hblk, 0, g.s, Ao, T, (int)GF_PS, 0, (int)GF_TSO);
+        wd_launch(hop_group_kernel<PS, 12, false, CG_NORM>, hgrid, hblk, 0, g.s, Ae, T, (int)GF_TSO, (int)GF_PS, (int)GF_TSE);
+        wd_launch(hop_group_kernel<PS, 12, true, CG_ALPHA>, hgrid_sum, hblk, 0, g.s, Ao, T, (int)GF_TSE, 0, (int)GF_TSO);
+        wd_launch(hop_group_kernel<PS, 12, true, CG_RESID>, hgrid, hblk, 0, g.s, Ae, T, (int)GF_TSO, (int)GF_TSE, 0);
     } else {
-        wd_launch(hop_group_kernel<PS, 18, false, false>, hgrid, hblk, 0, g.s, Ao, T, (int)GF_PS, 0, (int)GF_TSO);
-        wd_launch(hop_group_kernel<PS, 18, false, true>, hgrid, hblk, 0, g.s, Ae, T, (int)GF_TSO, (int)GF_PS, (int)GF_TSE);
-        wd_launch(hop_group_kernel<PS, 18, true, false>, hgrid, hblk, 0, g.s, Ao, T, (int)GF_TSE, 0, (int)GF_TSO);
-        wd_launch(hop_group_kernel<PS, 18, true, true>, hgrid, hblk, 0, g.s, Ae, T, (int)GF_TSO, (int)GF_TSE, (int)GF_APS);
+        wd_launch(hop_group_kernel<PS, 18, false, 0>, hgrid, hblk, 0, g.s, Ao, T, (int)GF_PS, 0, (int)GF_TSO);
+        wd_launch(hop_group_kernel<PS, 18, false, CG_NORM>, hgrid, hblk, 0, g.s, Ae, T, (int)GF_TSO, (int)GF_PS, (int)GF_TSE);
+        wd_launch(hop_group_kernel<PS, 18, true, CG_ALPHA>, hgrid_sum, hblk, 0, g.s, Ao, T, (int)GF_TSE, 0, (int)GF_TSO);
+        wd_launch(hop_group_kernel<PS, 18, true, CG_RESID>, hgrid, hblk, 0, g.s, Ae, T, (int)GF_TSO, (int)GF_TSE, 0);
     }
-    wd_launch(gg_dot_kernel<PS>, bgrid, bblk, 0, g.s, T, vh);
-    wd_launch(gg_update_kernel<PS>, bgrid, bblk, 0, g.s, T, vh);
-    wd_launch(gg_control_kernel, dim3(1), dim3(GG_MAX), 0, g.s, g.d_table, g.d_hs, g.cond);
+    wd_launch(gg_control_kernel, dim3((unsigned)cg_parts(vh, BLAS_THREADS), (unsigned)GG_BLAS_ROWS), bblk, 0, g.s,
+              g.d_table, g.d_hs, vh, g.cond);
     graph_sink() = nullptr;
     if (sink.err != cudaSuccess) {
         cudaGraphDestroy(graph);
@@ -323,9 +333,9 @@ inline GMember gg_member(const GSolve &q)
     GMember m{};
     m.f[GF_RS] = q.rs;
     m.f[GF_PS] = q.ps;
-    m.f[GF_APS] = q.aps;
     m.f[GF_TSO] = q.tso;
     m.f[GF_TSE] = q.tse;
+    m.site = q.site;
     m.xs = q.xs;
     m.scal = q.scal;
     m.red = q.red;
@@ -341,6 +351,7 @@ inline int gg_launch(GGroup &g, const int *slots, int n)
 {
     g.h_table->n = n;
     g.h_table->launch_iters = 0;
+    g.h_table->done = g.h_table->stop = 0;
     for (int k = 0; k < n; ++k) g.h_table->idx[k] = slots[k];
     WD_CUDA_TRY(cudaMemcpyAsync(g.d_table, g.h_table, sizeof(GTable), cudaMemcpyHostToDevice, g.s));
     WD_CUDA_TRY(cudaGraphLaunch(g.exec, g.s));

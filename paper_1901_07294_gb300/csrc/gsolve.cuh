@@ -4,8 +4,9 @@
 // Shared by the graph batch mode and the request queue.  A solve owns its
 // workspace, a stream, per-solve reduction scratch and a graph whose only
 // top-level node is a conditional WHILE node.  Its body is one CG iteration
-// (4 hop launches and 3 BLAS kernels, every CG scalar in device memory)
-// followed by a one-thread control kernel that tracks max |r| and the
+// (the update of x and p, then 4 hop launches that carry the step length and
+// the residual update, dslash_cg.cuh; every CG scalar in device memory)
+// followed by a control kernel that adds up |r|^2, tracks max |r| and the
 // iteration counts and keeps the loop going until a reliable update is due
 // (|r| < delta max|r|, |r|^2 <= tol^2 |b|^2, a breakdown, RELIABLE_MAX_GAP
 // iterations without an update, maxiter) or GS_LAUNCH_CAP iterations have run
@@ -19,13 +20,16 @@
 #include <cstring>
 
 #include "blas_host.cuh"
+#include "cg_iter.h"
+#include "dslash_cg.cuh"
 
 namespace wd {
 
 constexpr int GS_LAUNCH_CAP = 32;   // iterations at most per graph launch
 
-// Device scalar slots of a graph-driven solve (see also OpDotAlphaDev):
-// s[0] |r|^2, s[1] pAp, s[2] alpha, s[3] true |r|^2, s[4] previous |r|^2,
+// Device scalar slots of a graph-driven solve: s[0] |r|^2, s[1] <p, A p>,
+// s[2] alpha of the last iteration, whose step is not yet in x (0: none
+// pending), s[3] true |r|^2, s[4] previous |r|^2,
 // s[5] beta = s[0] / s[4] for the next direction update, s[6] breakdown flag, s[8] max |r| since the last update, s[9] iterations in
 // this launch, s[10] iterations since the last update, s[11] iterations in
 // total, s[12] tol^2 |b|^2, s[13] delta, s[14] maxiter, s[15] GS_LAUNCH_CAP.
@@ -47,18 +51,23 @@ __device__ __forceinline__ bool gs_member_step(double *s)
     s[10] = n_gap;
     s[11] = n_total;
     const bool finite = r2 == r2 && r2 < 1e300;
-    s[5] = s[4] > 0.0 ? r2 / s[4] : 0.0;   // once here, not per site in OpXpayDev
+    s[5] = s[4] > 0.0 ? r2 / s[4] : 0.0;   // read by the next direction update (OpXp)
     return s[6] != 0.0 || !finite || rn < s[13] * maxr || r2 <= s[12] || n_total >= s[14] ||
            n_gap >= (double)RELIABLE_MAX_GAP || n_launch >= s[15];
 }
 
-// The loop condition of the WHILE node, evaluated after each iteration.
+// The end of an iteration: |r|^2 from its site sums, the bookkeeping and the
+// loop condition of the WHILE node.
 template <int UNUSED = 0>
-__global__ void gs_control_kernel(double *s, cudaGraphConditionalHandle cond)
+__global__ void __launch_bounds__(256)
+    gs_control_kernel(double *s, const float *site, int n, RedScratch red, cudaGraphConditionalHandle cond)
 {
     grid_dependency_enter();
-    if (threadIdx.x != 0) return;
-    cudaGraphSetConditional(cond, gs_member_step(s) ? 0u : 1u);
+    site_sum(site, n, blockIdx.x, gridDim.x, red, [&](double v) {
+        s[4] = s[0];
+        s[0] = v;
+        cudaGraphSetConditional(cond, gs_member_step(s) ? 0u : 1u);
+    });
 }
 
 struct GSolve {
@@ -76,8 +85,9 @@ struct GSolve {
     void *mem = nullptr;
     double *h = nullptr;   // pinned host copy of the scalars
     char *r = nullptr, *ax = nullptr, *t_o = nullptr, *t_e = nullptr;
-    char *rs = nullptr, *ps = nullptr, *aps = nullptr, *tso = nullptr, *tse = nullptr, *xs = nullptr;
-    double *scal = nullptr;   // device scalars, see OpDotAlphaDev
+    char *rs = nullptr, *ps = nullptr, *tso = nullptr, *tse = nullptr, *xs = nullptr;
+    float *site = nullptr;    // per-site sums
+    double *scal = nullptr;   // device scalars (slots above)
     RedScratch red{};
     // state
     double b2 = 0, stop2 = 0, maxr = 0;
@@ -118,8 +128,9 @@ template <typename Op> inline int launch(const wd_ctx *ctx, const Op &op, int ns
     return e == cudaSuccess ? WD_OK : set_error(WD_ECUDA, "BLAS launch failed: %s", cudaGetErrorString(e));
 }
 
-// One iteration, starting with the direction update p = r + beta p
-// (beta = s[5] = s[0]/s[4]; s[4] = +inf, s[5] = 0 give p = r).  A launch therefore ends right
+// One iteration, starting with the updates x += alpha p (the step of the last
+// iteration; alpha = s[2], 0 if none is pending) and p = r + beta p (beta =
+// s[5] = s[0]/s[4]; s[4] = +inf, s[5] = 0 give p = r).  A launch therefore ends right
 // after a residual update, and a host-side reliable update that replaces r
 // and s[0] between launches is picked up by the next direction update, as in
 // the sequential solver.
@@ -127,14 +138,10 @@ template <int PS> int iteration(const wd_ctx *ctx, GSolve &q)
 {
     const int vh = q.vh;
     auto FS = [&](const void *p) { return field_ref<PS>(p, vh); };
-    auto FX = [&](const void *p) { return field_ref<PREC_F32>(p, vh); };
-    WD_TRY(launch(ctx, OpXpayDev<PS>{FS(q.rs), FS(q.ps), q.scal}, vh, q.red, q.s));
-    WD_TRY(mdagm(q.gauge, PS, q.opts.inner_recon, q.mass, q.ps, q.aps, q.tso, q.tse, q.s));
-    WD_TRY(launch(ctx, OpDotAlphaDev<PS>{FS(q.ps), FS(q.aps), q.scal}, vh, q.red, q.s));
-    OpCgUpdateDev<PREC_F32, PS> up{
-        OpCgUpdate<PREC_F32, PS>{FX(q.xs), FS(q.rs), FS(q.ps), FS(q.aps), q.scal + 2, nullptr}, q.scal};
-    WD_TRY(launch(ctx, up, vh, q.red, q.s));
-    return WD_OK;
+    WD_TRY(launch(ctx, OpXp<PREC_F32, PS>{field_ref<PREC_F32>(q.xs, vh), FS(q.rs), FS(q.ps), q.scal + 2, q.scal + 5, 0.0},
+                  vh, q.red, q.s));
+    return cg_iteration_hops(q.gauge, PS, q.opts.inner_recon, q.mass,
+                             CgFields{q.ps, q.rs, q.tso, q.tse, q.site, q.scal, q.red.partials, q.red.ticket}, q.s);
 }
 
 // r = b - A x (FP64; A applied in precision op, FP64 or double-word FP32);
@@ -153,14 +160,14 @@ template <int PS> int residual_reseed(const wd_ctx *ctx, GSolve &q, int op)
     return WD_OK;
 }
 
-// x += x_lo, then residual_reseed in FP64 or the solve's outer precision (q.update_fp64).
+// x += x_lo and the step still pending, then residual_reseed in FP64 or the
+// solve's outer precision (q.update_fp64).
 template <int PS> int reliable_update(const wd_ctx *ctx, GSolve &q)
 {
     const int vh = q.vh;
-    auto F64 = [&](const void *p) { return field_ref<PREC_F64>(p, vh); };
-    auto FX = [&](const void *p) { return field_ref<PREC_F32>(p, vh); };
-    WD_TRY(launch(ctx, OpAxpby<PREC_F32, PREC_F64>{FX(q.xs), F64(q.x), 1.0, 1.0}, vh, q.red, q.s));
-    WD_CUDA_TRY(cudaMemsetAsync(q.xs, 0, half_field_bytes(vh, WD_F32), q.s));
+    WD_TRY(launch(ctx, OpFlushX<PREC_F32, PS>{field_ref<PREC_F64>(q.x, vh), field_ref<PREC_F32>(q.xs, vh),
+                                              field_ref<PS>(q.ps, vh), q.scal + 2}, vh, q.red, q.s));
+    WD_CUDA_TRY(cudaMemsetAsync(q.scal + 2, 0, sizeof(double), q.s));
     return residual_reseed<PS>(ctx, q, q.update_fp64 ? WD_F64 : outer_prec_of(q.opts));
 }
 
@@ -199,7 +206,8 @@ template <int PS> int init(const wd_ctx *ctx, GSolve &q, bool with_graph)
     sink.graph = cp.conditional.phGraph_out[0];
     graph_sink() = &sink;
     int rc = iteration<PS>(ctx, q);
-    if (rc == WD_OK && wd_launch(gs_control_kernel<0>, dim3(1), dim3(32), 0, q.s, q.scal, q.cond) != cudaSuccess)
+    if (rc == WD_OK && wd_launch(gs_control_kernel<0>, dim3(cg_parts(vh, 256)), dim3(256), 0, q.s, q.scal,
+                                 (const float *)q.site, vh, q.red, q.cond) != cudaSuccess)
         rc = set_error(WD_ECUDA, "adding the loop control failed");
     graph_sink() = nullptr;
     if (rc == WD_OK && sink.err != cudaSuccess)
@@ -261,7 +269,7 @@ inline int gs_bind(const wd_ctx *ctx, GSolve &q, bool graph = true)
     };
     const size_t h64 = (size_t)q.vh * 192, hs = half_field_bytes(q.vh, q.prec);
     q.r = take(h64); q.ax = take(h64); q.t_o = take(h64); q.t_e = take(h64);
-    q.rs = take(hs); q.ps = take(hs); q.aps = take(hs); q.tso = take(hs); q.tse = take(hs);
+    q.rs = take(hs); q.ps = take(hs); q.site = (float *)take(hs); q.tso = take(hs); q.tse = take(hs);
     q.xs = take((size_t)q.vh * 96);
     q.scal = (double *)take(256);
     q.red.ticket = (unsigned *)take(256);
