@@ -23,8 +23,8 @@ constexpr int DF_ROW_BLOCKS = 8;   // resident blocks per SM the register budget
 
 // (h0, h1) = upper two spin components of (1 + S gamma_MU) psi for one colour,
 // from its four spin components p[s] (the table of project).
-template <int MU, int S>
-__device__ __forceinline__ void project_colour(const cpx<df> (&p)[4], cpx<df> &h0, cpx<df> &h1)
+template <int MU, int S, typename T>
+__device__ __forceinline__ void project_colour(const cpx<T> (&p)[4], cpx<T> &h0, cpx<T> &h1)
 {
     if constexpr (MU == 0) {        // h0 = p0 + S i p3, h1 = p1 + S i p2
         h0 = {p[0].re - S * p[3].im, p[0].im + S * p[3].re};

@@ -476,12 +476,9 @@ __device__ __forceinline__ void hop_site(const HopArgs &A, const int p, const in
 
 // PF 4 is schedule 1 compiled for 3 resident blocks of 256 threads per SM
 // (at most 85 registers): more warps to hide latency, at the price of
-// registers the compiler would otherwise use to hoist loads.  PF 5 is
-// schedule 0 compiled for one block of 256 per SM: the FP64 kernel, bound by
-// the FP64 pipe rather than by latency, then needs no spill stores (at the
-// 128-register cap of two blocks it spills 200-550 bytes per thread).  PF 6
-// is schedule 1 compiled the same way (double-word FP32, whose values take
-// two registers like FP64 ones).
+// registers the compiler would otherwise use to hoist loads.  PF 5 and 6 are
+// schedules 0 and 1 compiled for one block of 256 per SM: double-word FP32,
+// whose values take two registers.
 template <int P, int RECON, bool DAG, bool HAS_X, int PF, bool TOPEN = false, bool LNA = false>
 __global__ void __launch_bounds__(256, PF == 4 ? 3 : (PF == 5 || PF == 6) ? 1 : 2) hop_kernel(const HopArgs A)
 {
@@ -506,9 +503,6 @@ cudaError_t launch_hop_pf(const HopArgs &A, dim3 grid, int threads, int pf, bool
     case 0: return wd_launch(hop_kernel<P, RECON, DAG, HX, 0>, grid, dim3(threads), 0, s, A);
     case 1: return wd_launch(hop_kernel<P, RECON, DAG, HX, 1>, grid, dim3(threads), 0, s, A);
     case 2: return wd_launch(hop_kernel<P, RECON, DAG, HX, 2>, grid, dim3(threads), 0, s, A);
-    case 5:
-        if constexpr (P == PREC_F64) return wd_launch(hop_kernel<P, RECON, DAG, HX, 5>, grid, dim3(threads), 0, s, A);
-        else return wd_launch(hop_kernel<P, RECON, DAG, HX, 0>, grid, dim3(threads), 0, s, A);
     default: return wd_launch(hop_kernel<P, RECON, DAG, HX, 4>, grid, dim3(threads), 0, s, A);
     }
 }

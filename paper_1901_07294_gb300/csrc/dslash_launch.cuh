@@ -3,6 +3,7 @@
 #pragma once
 
 #include "dslash_df.cuh"
+#include "dslash_f64.cuh"
 #include "dslash_impl.cuh"
 #include "dslash_mrhs.cuh"
 #include "dslash_pair.cuh"
@@ -20,7 +21,7 @@ constexpr int HOP_NA0_VARIANT = 11;   // schedule 0 with the links loaded withou
 constexpr int HOP_NA1_VARIANT = 12;   // schedule 1 with the links loaded without L1 allocation
 constexpr int HOP_SP1_VARIANT = 13;   // 16-bit formats: schedule 1 with spin-paired FP32 arithmetic
 constexpr int HOP_SP0_VARIANT = 14;   // 16-bit formats: schedule 0, spin-paired, links without L1 allocation
-constexpr int HOP_F64_1B_VARIANT = 15;// FP64: schedule 0 built for one block of 256 per SM (no spills); else schedule 0
+constexpr int HOP_ROW_VARIANT = 15;   // FP64 and double-word: three threads per site (its own block shape); else schedule 0
 constexpr int HOP_MAX_VARIANT = 15;   // 5, 6, 7: the multi-RHS kernel in z-strips of 16, 8, 4
 
 // Multi-RHS variants and their z-strip width (0: natural order); -1 if v is not one.
@@ -88,7 +89,21 @@ cudaError_t launch_hop_std(const HopArgs &A, int nrhs, int threads, int pf, int 
     }
     if (pf == HOP_SP1_VARIANT) pf = 1;   // FP32, FP64, or an open-boundary pass
     if (pf == HOP_SP0_VARIANT) pf = 0;
-    if (pf == HOP_F64_1B_VARIANT) pf = 5;   // launch_hop_pf: schedule 0 outside FP64
+    if constexpr (P == PREC_F64) {
+        if (pf == HOP_ROW_VARIANT && !A.topen) {
+            switch (key) {
+            case 0: return launch_hop_f64_row<18, false, false>(A, nrhs, s);
+            case 1: return launch_hop_f64_row<18, false, true>(A, nrhs, s);
+            case 2: return launch_hop_f64_row<18, true, false>(A, nrhs, s);
+            case 3: return launch_hop_f64_row<18, true, true>(A, nrhs, s);
+            case 4: return launch_hop_f64_row<12, false, false>(A, nrhs, s);
+            case 5: return launch_hop_f64_row<12, false, true>(A, nrhs, s);
+            case 6: return launch_hop_f64_row<12, true, false>(A, nrhs, s);
+            default: return launch_hop_f64_row<12, true, true>(A, nrhs, s);
+            }
+        }
+    }
+    if (pf == HOP_ROW_VARIANT) pf = 0;   // FP32, the 16-bit formats, or an open-boundary pass
     cudaError_t e = cudaSuccess;
     if (pf == HOP_RETIRED_VARIANT) pf = 1;
     if (pf == HOP_TILE_VARIANT) {
@@ -131,12 +146,12 @@ cudaError_t launch_hop(const HopArgs &A, int recon, int dagger, int nrhs, int th
     const bool hx = A.x[0] != nullptr || A.x[1] != nullptr;
     const int key = (recon == 12 ? 4 : 0) + (dagger ? 2 : 0) + (hx ? 1 : 0);
     if constexpr (P == PREC_DF) {
-        // double-word FP32: variant HOP_F64_1B_VARIANT is the
+        // double-word FP32: variant HOP_ROW_VARIANT is the
         // three-threads-per-site kernel (dslash_df.cuh); otherwise one site
         // per thread, one block of 256 per SM, schedule 1 for variants 1 and 12
         // and schedule 0 for the rest
         if (A.topen) return cudaErrorInvalidValue;
-        if (pf == HOP_F64_1B_VARIANT) {
+        if (pf == HOP_ROW_VARIANT) {
             switch (key) {
             case 0: return launch_hop_df_row<18, false, false>(A, nrhs, s);
             case 1: return launch_hop_df_row<18, false, true>(A, nrhs, s);

@@ -99,6 +99,52 @@ cudaError_t wd_launch(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t sm
     return e;
 }
 
+// SMs of the current device (queried once per device).
+inline int device_sm_count()
+{
+    static std::atomic<int> cache[64] = {};
+    int dev = -1;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 152;
+    int v = cache[dev].load(std::memory_order_relaxed);
+    if (v == 0) {
+        if (cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || v <= 0) {
+            cudaGetLastError();
+            v = 152;
+        }
+        cache[dev].store(v, std::memory_order_relaxed);
+    }
+    return v;
+}
+
+// Dynamic shared memory that keeps a grid of less than a full wave evenly
+// spread.  A kernel dispatched while its predecessor's last blocks run finds
+// some SMs free and fills them to their limit, so a grid of, say, 6.7 blocks per
+// SM of a kernel that fits 8 ends up with 8 on some SMs and the others idle; asking for so
+// much shared memory that only ceil(blocks / SMs) fit gives every SM its share.
+// 0 if the grid fills the device anyway.
+inline size_t spread_smem(long long blocks, int resident, size_t static_bytes)
+{
+    const long long sms = device_sm_count(), k = (blocks + sms - 1) / sms;
+    if (k >= resident || k < 1) return 0;
+    const size_t per = (size_t)228 * 1024 / (size_t)k - 1024;   // 1 KB of each block's share is the system's
+    const size_t most = 227 * 1024;
+    return (per < most ? per : most) - static_bytes;
+}
+
+// Lets `kernel` use up to 227 KB of dynamic shared memory (less its static
+// part), once per kernel and device.
+template <typename K> inline cudaError_t allow_smem(K *kernel, std::atomic<unsigned long long> &done, size_t static_bytes)
+{
+    int dev = -1;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    const unsigned long long bit = 1ull << (dev & 63);
+    if (done.load(std::memory_order_acquire) & bit) return cudaSuccess;
+    e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(227 * 1024 - static_bytes));
+    if (e == cudaSuccess) done.fetch_or(bit, std::memory_order_release);
+    return e;
+}
+
 // SM clock of device `dev` (-1: the current one) in kHz, queried once per
 // device: the query takes hundreds of microseconds, far longer than a launch.
 // Used to turn the bounded waits' limits from seconds into clock cycles.
