@@ -215,6 +215,19 @@ __device__ __forceinline__ uint4 ldg16_na(const void *p)
 }
 __device__ __forceinline__ void stg16(void *p, uint4 v) { *reinterpret_cast<uint4 *>(p) = v; }
 
+// Asynchronous copy of N = 4, 8 or 16 bytes from global to shared memory by
+// this thread (both addresses N-byte aligned); it needs no registers while in
+// flight.  NA: without L1 allocation (16 bytes only).  A thread's copies are
+// grouped by copy_commit; copy_wait<N> waits until at most its N latest groups
+// are in flight, after which it may read what its earlier groups brought.
+template <int N, bool NA = false> __device__ __forceinline__ void copy_async(unsigned dst, const void *src)
+{
+    if constexpr (NA && N == 16) asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
+    else asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"(dst), "l"(src), "n"(N) : "memory");
+}
+__device__ __forceinline__ void copy_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N> __device__ __forceinline__ void copy_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
+
 // Hint: bring the 128-byte line holding p into L2 (no register result).
 __device__ __forceinline__ void prefetch_l2(const void *p)
 {
