@@ -112,6 +112,57 @@ __device__ __forceinline__ void hop_dir_smem(const char *in, int vh, int nb,
     accumulate<MU, S>(acc, w0, w1);
 }
 
+// The eight directions of one site and field, links from the tile (`lk`: the
+// first vector of direction 0 at the site's column), neighbour indices nb[32 d].
+// Neighbours along +x and -x (and +y, -y) share most of their cache lines within a
+// warp, so PAIRS takes each pair in a row; otherwise backward directions
+// first.  FP32 (12 fields, even-odd, 32^4) 380 us backward first, 372 in pairs;
+// FP16 on 16^3 x 32 46.0 and 46.7 us.
+template <int P, int SF, bool PAIRS>
+__device__ __forceinline__ void hop_site_smem(const char *in, int vh, int i, const int *nb,
+                                              const typename LinkTile<typename Prec<P>::real>::V *lk, bool tneg,
+                                              const float wt, cpx<typename Prec<P>::real> (&acc)[4][3])
+{
+    using T = typename Prec<P>::real;
+    constexpr int SB = -SF, D = LinkTile<T>::NV * 32;   // vectors of one direction
+    const bool ntf = tneg && nb[96] < i, ntb = tneg && nb[224] > i;
+#pragma unroll
+    for (int sp = 0; sp < 4; ++sp)
+#pragma unroll
+        for (int c = 0; c < 3; ++c) acc[sp][c] = {T(0), T(0)};
+    if constexpr (PAIRS) {
+        hop_dir_smem<P, 0, SB, false>(in, vh, nb[128], lk + 4 * D, false, acc, wt);
+        hop_dir_smem<P, 0, SF, true>(in, vh, nb[0], lk, false, acc, wt);
+        hop_dir_smem<P, 1, SB, false>(in, vh, nb[160], lk + 5 * D, false, acc, wt);
+        hop_dir_smem<P, 1, SF, true>(in, vh, nb[32], lk + 1 * D, false, acc, wt);
+        hop_dir_smem<P, 2, SB, false>(in, vh, nb[192], lk + 6 * D, false, acc, wt);
+        hop_dir_smem<P, 2, SF, true>(in, vh, nb[64], lk + 2 * D, false, acc, wt);
+        hop_dir_smem<P, 3, SB, false>(in, vh, nb[224], lk + 7 * D, ntb, acc, wt);
+        hop_dir_smem<P, 3, SF, true>(in, vh, nb[96], lk + 3 * D, ntf, acc, wt);
+    } else {
+        hop_dir_smem<P, 0, SB, false>(in, vh, nb[128], lk + 4 * D, false, acc, wt);
+        hop_dir_smem<P, 1, SB, false>(in, vh, nb[160], lk + 5 * D, false, acc, wt);
+        hop_dir_smem<P, 2, SB, false>(in, vh, nb[192], lk + 6 * D, false, acc, wt);
+        hop_dir_smem<P, 3, SB, false>(in, vh, nb[224], lk + 7 * D, ntb, acc, wt);
+        hop_dir_smem<P, 0, SF, true>(in, vh, nb[0], lk, false, acc, wt);
+        hop_dir_smem<P, 1, SF, true>(in, vh, nb[32], lk + 1 * D, false, acc, wt);
+        hop_dir_smem<P, 2, SF, true>(in, vh, nb[64], lk + 2 * D, false, acc, wt);
+        hop_dir_smem<P, 3, SF, true>(in, vh, nb[96], lk + 3 * D, ntf, acc, wt);
+    }
+}
+
+// A grid of shared-link blocks (`threads` threads each) that is at most two waves
+// of the 128-register build: short launches gain more from a thread with its
+// loads in flight than from more warps (80 registers: half again as many).  us, 80
+// against 128 registers, direction pairs: 16^4 even-odd, 6 FP16 fields 15.0 / 12.8,
+// 8 FP32 fields 21.7 / 18.9; 8^2 x 16^2 full, 12 FP16 fields 17.5 / 12.5; 8^4
+// even-odd, 12 FP32 fields 7.9 / 6.5; beyond two waves the other way: 16^3 x 32
+// even-odd, 6 FP16 fields 22.6 / 24.2, full 46.7 / 52.3; 32^4, 12 FP32 fields 372 / 390.
+inline bool mrhs_small(long long blocks, int threads)
+{
+    return blocks * threads <= 2LL * 512 * device_sm_count();
+}
+
 // out = a x + b acc at site i of parity p for the field at byte offset roff
 template <int P, bool HAS_X>
 __device__ __forceinline__ void mrhs_store(const HopArgs &A, int p, int i, size_t roff,
@@ -151,9 +202,10 @@ __device__ __forceinline__ void mrhs_store(const HopArgs &A, int p, int i, size_
 // rebuilt once for 12-real storage) into shared memory, then warp y of the
 // block computes right-hand sides y, y + blockDim.y, ... from them, so links
 // cost 1/nrhs of their single-field traffic.  Spinors are read per field as in
-// hop_kernel.  blockDim = (32, RY).  Reduced precisions are compiled for 3
-// resident blocks of 256 threads per SM (at most 80 registers, no spills);
-// FP64 needs twice the registers per complex number and is left unbounded.
+// hop_kernel.  blockDim = (32, RY).  MINB: resident blocks of 256 threads per SM
+// the kernel is compiled for: 3 (at most 80 registers, no spills) or, for small
+// grids (mrhs_small), 2; FP64 needs twice the registers per complex number and is
+// left unbounded (1).
 //
 // Site order.  With zs = 0 block b takes checkerboard sites 32b .. 32b+31, so
 // the (z, t) slices of the lattice are visited t-major and a source spinor read
@@ -180,8 +232,8 @@ __device__ __forceinline__ int mrhs_site(const HopArgs &A, int j, int zs)
     return off + sxy * (z + A.L[2] * t);
 }
 
-template <int P, int RECON, bool DAG, bool HAS_X>
-__global__ void __launch_bounds__(256, P == PREC_F64 ? 1 : 3) hop_mrhs_kernel(const HopArgs A, const int nrhs, const int zs)
+template <int P, int RECON, bool DAG, bool HAS_X, int MINB>
+__global__ void __launch_bounds__(256, MINB) hop_mrhs_kernel(const HopArgs A, const int nrhs, const int zs)
 {
     grid_dependency_enter();
     using T = typename Prec<P>::real;
@@ -231,24 +283,12 @@ __global__ void __launch_bounds__(256, P == PREC_F64 ? 1 : 3) hop_mrhs_kernel(co
                                   // (t = Lt-1 forward, t = 0 backward) exactly when that
                                   // neighbour's checkerboard index falls below / above i
     constexpr int SF = DAG ? +1 : -1;
-    constexpr int SB = -SF;
     for (int rhs = threadIdx.y; rhs < nrhs; rhs += blockDim.y) {
         const size_t roff = (size_t)rhs * A.rhs_stride;
         const char *in = (p ? A.in[1] : A.in[0]) + roff;
         const float wt = Prec<P>::scaled ? (float)A.b : 1.0f;   // 16-bit: b weights the terms
         cpx<T> acc[4][3];
-#pragma unroll
-        for (int sp = 0; sp < 4; ++sp)
-#pragma unroll
-            for (int c = 0; c < 3; ++c) acc[sp][c] = {T(0), T(0)};
-        hop_dir_smem<P, 0, SB, false>(in, vh, nb[128], &lk[4][0][s], false, acc, wt);
-        hop_dir_smem<P, 1, SB, false>(in, vh, nb[160], &lk[5][0][s], false, acc, wt);
-        hop_dir_smem<P, 2, SB, false>(in, vh, nb[192], &lk[6][0][s], false, acc, wt);
-        hop_dir_smem<P, 3, SB, false>(in, vh, nb[224], &lk[7][0][s], A.tneg && nb[224] > i, acc, wt);
-        hop_dir_smem<P, 0, SF, true>(in, vh, nb[0], &lk[0][0][s], false, acc, wt);
-        hop_dir_smem<P, 1, SF, true>(in, vh, nb[32], &lk[1][0][s], false, acc, wt);
-        hop_dir_smem<P, 2, SF, true>(in, vh, nb[64], &lk[2][0][s], false, acc, wt);
-        hop_dir_smem<P, 3, SF, true>(in, vh, nb[96], &lk[3][0][s], A.tneg && nb[96] < i, acc, wt);
+        hop_site_smem<P, SF, MINB == 2 || !Prec<P>::scaled>(in, vh, i, nb, &lk[0][0][s], A.tneg, wt, acc);
         mrhs_store<P, HAS_X>(A, p, i, roff, acc);
     }
 }
@@ -259,7 +299,11 @@ cudaError_t launch_hop_mrhs(const HopArgs &A, int nrhs, int threads, int zs, cud
     const int ry = threads / 32;
     const int per = (A.vh + 31) / 32;
     if (zs <= 0 || zs >= A.L[2]) zs = 0;
-    return wd_launch(hop_mrhs_kernel<P, RECON, DAG, HX>, dim3((unsigned)(per * A.nparity)), dim3(32, ry), 0, s, A, nrhs, zs);
+    const dim3 grid((unsigned)(per * A.nparity)), block(32, ry);
+    if constexpr (P == PREC_F64) return wd_launch(hop_mrhs_kernel<P, RECON, DAG, HX, 1>, grid, block, 0, s, A, nrhs, zs);
+    else if (mrhs_small(grid.x, threads))
+        return wd_launch(hop_mrhs_kernel<P, RECON, DAG, HX, 2>, grid, block, 0, s, A, nrhs, zs);
+    else return wd_launch(hop_mrhs_kernel<P, RECON, DAG, HX, 3>, grid, block, 0, s, A, nrhs, zs);
 }
 
 } // namespace wd

@@ -69,8 +69,10 @@ struct GTable {
 constexpr int GG_SUM_THREADS = 128;   // threads of a hop block
 constexpr int GG_SUM_BLOCKS = 64;   // blocks of a CG_ALPHA launch that add site sums
 
-template <int P, int RECON, bool DAG, int STEP>
-__global__ void __launch_bounds__(128, 6)
+// SMALL: the build for small lattices (mrhs_small of the lattice alone, so that a
+// member's arithmetic does not depend on the group).
+template <int P, int RECON, bool DAG, int STEP, bool SMALL>
+__global__ void __launch_bounds__(128, SMALL ? 4 : 6)
     hop_group_kernel(const HopArgs A, const GTable *__restrict__ T, const int fi, const int fx, const int fo)
 {
     grid_dependency_enter();
@@ -131,25 +133,13 @@ __global__ void __launch_bounds__(128, 6)
     if (!active) return;
     const int *nb = &nbs[0][s];
     constexpr int SF = DAG ? +1 : -1;
-    constexpr int SB = -SF;
     for (int r = threadIdx.y; r < n; r += blockDim.y) {
         const GMember &m = T->m[T->idx[r]];
         const char *in = m.f[fi];
         // 16-bit: the member's hop coefficient weights the terms
         const float wt = Prec<P>::scaled && HAS_X ? (float)m.mc : 1.0f;
         cpx<T_> acc[4][3];
-#pragma unroll
-        for (int sp = 0; sp < 4; ++sp)
-#pragma unroll
-            for (int c = 0; c < 3; ++c) acc[sp][c] = {T_(0), T_(0)};
-        hop_dir_smem<P, 0, SB, false>(in, vh, nb[128], &lk[4][0][s], false, acc, wt);
-        hop_dir_smem<P, 1, SB, false>(in, vh, nb[160], &lk[5][0][s], false, acc, wt);
-        hop_dir_smem<P, 2, SB, false>(in, vh, nb[192], &lk[6][0][s], false, acc, wt);
-        hop_dir_smem<P, 3, SB, false>(in, vh, nb[224], &lk[7][0][s], A.tneg && nb[224] > i, acc, wt);
-        hop_dir_smem<P, 0, SF, true>(in, vh, nb[0], &lk[0][0][s], false, acc, wt);
-        hop_dir_smem<P, 1, SF, true>(in, vh, nb[32], &lk[1][0][s], false, acc, wt);
-        hop_dir_smem<P, 2, SF, true>(in, vh, nb[64], &lk[2][0][s], false, acc, wt);
-        hop_dir_smem<P, 3, SF, true>(in, vh, nb[96], &lk[3][0][s], A.tneg && nb[96] < i, acc, wt);
+        hop_site_smem<P, SF, SMALL>(in, vh, i, nb, &lk[0][0][s], A.tneg, wt, acc);
         T_ o[24];
         if constexpr (Prec<P>::scaled) {
             value_weighted<P, HAS_X>(HAS_X ? m.f[fx] : nullptr, vh, i, (float)m.ma, acc, o);
@@ -273,17 +263,21 @@ template <int PS> int build(const wd_ctx *ctx, GGroup &g)
     Ae.parity0 = WD_EVEN;
     const dim3 hgrid_sum(hgrid.x + GG_SUM_BLOCKS);
     wd_launch(gg_xp_kernel<PS>, bgrid, bblk, 0, g.s, T, vh);
-    if (g.recon == 12) {
-        wd_launch(hop_group_kernel<PS, 12, false, 0>, hgrid, hblk, 0, g.s, Ao, T, (int)GF_PS, 0, (int)GF_TSO);
-        wd_launch(hop_group_kernel<PS, 12, false, CG_NORM>, hgrid, hblk, 0, g.s, Ae, T, (int)GF_TSO, (int)GF_PS, (int)GF_TSE);
-        wd_launch(hop_group_kernel<PS, 12, true, CG_ALPHA>, hgrid_sum, hblk, 0, g.s, Ao, T, (int)GF_TSE, 0, (int)GF_TSO);
-        wd_launch(hop_group_kernel<PS, 12, true, CG_RESID>, hgrid, hblk, 0, g.s, Ae, T, (int)GF_TSO, (int)GF_TSE, 0);
-    } else {
-        wd_launch(hop_group_kernel<PS, 18, false, 0>, hgrid, hblk, 0, g.s, Ao, T, (int)GF_PS, 0, (int)GF_TSO);
-        wd_launch(hop_group_kernel<PS, 18, false, CG_NORM>, hgrid, hblk, 0, g.s, Ae, T, (int)GF_TSO, (int)GF_PS, (int)GF_TSE);
-        wd_launch(hop_group_kernel<PS, 18, true, CG_ALPHA>, hgrid_sum, hblk, 0, g.s, Ao, T, (int)GF_TSE, 0, (int)GF_TSO);
-        wd_launch(hop_group_kernel<PS, 18, true, CG_RESID>, hgrid, hblk, 0, g.s, Ae, T, (int)GF_TSO, (int)GF_TSE, 0);
-    }
+    auto hops = [&](auto recon, auto small) {
+        constexpr int R = decltype(recon)::value;
+        constexpr bool S = decltype(small)::value;
+        wd_launch(hop_group_kernel<PS, R, false, 0, S>, hgrid, hblk, 0, g.s, Ao, T, (int)GF_PS, 0, (int)GF_TSO);
+        wd_launch(hop_group_kernel<PS, R, false, CG_NORM, S>, hgrid, hblk, 0, g.s, Ae, T, (int)GF_TSO, (int)GF_PS,
+                  (int)GF_TSE);
+        wd_launch(hop_group_kernel<PS, R, true, CG_ALPHA, S>, hgrid_sum, hblk, 0, g.s, Ao, T, (int)GF_TSE, 0,
+                  (int)GF_TSO);
+        wd_launch(hop_group_kernel<PS, R, true, CG_RESID, S>, hgrid, hblk, 0, g.s, Ae, T, (int)GF_TSO, (int)GF_TSE, 0);
+    };
+    using R12 = std::integral_constant<int, 12>;
+    using R18 = std::integral_constant<int, 18>;
+    const bool small = mrhs_small(hgrid.x, GG_SUM_THREADS);
+    if (g.recon == 12) small ? hops(R12{}, std::true_type{}) : hops(R12{}, std::false_type{});
+    else small ? hops(R18{}, std::true_type{}) : hops(R18{}, std::false_type{});
     wd_launch(gg_control_kernel, dim3((unsigned)cg_parts(vh, BLAS_THREADS), (unsigned)GG_BLAS_ROWS), bblk, 0, g.s,
               g.d_table, g.d_hs, vh, g.cond);
     graph_sink() = nullptr;
