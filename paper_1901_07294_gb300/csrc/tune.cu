@@ -50,6 +50,7 @@ void load_tune_file(wd_ctx *ctx)
             variant != HOP_RETIRED_VARIANT)
             ctx->tuned[key] = {threads, variant};
     }
+    ctx->any_tuned.store(!ctx->tuned.empty(), std::memory_order_release);
 }
 
 } // namespace wd
@@ -150,6 +151,7 @@ int wd_tune_dslash(wd_ctx *ctx, const wd_gauge *g, int prec, int recon, int full
     {
         std::lock_guard<std::mutex> lk(ctx->tune_mu);
         ctx->tuned[key] = {best_t, best_v};
+        ctx->any_tuned.store(true, std::memory_order_release);
         if (!ctx->tune_file.empty()) {
             FILE *f = std::fopen(ctx->tune_file.c_str(), "a");
             if (f) {
@@ -177,6 +179,7 @@ int wd_tune_set_dslash(wd_ctx *ctx, const wd_gauge *g, int prec, int recon, int 
     A.x[0] = A.x[1] = (full || with_x) ? &dummy : nullptr;
     std::lock_guard<std::mutex> lk(ctx->tune_mu);
     ctx->tuned[hop_key(ctx, A, prec, recon, nrhs)] = {threads, variant};
+    ctx->any_tuned.store(true, std::memory_order_release);
     return WD_OK;
 }
 
@@ -211,6 +214,7 @@ int wd_tune_clear(wd_ctx *ctx)
     if (!ctx) return set_error(WD_EINVAL, "ctx is NULL");
     std::lock_guard<std::mutex> lk(ctx->tune_mu);
     ctx->tuned.clear();
+    ctx->any_tuned.store(false, std::memory_order_release);
     return WD_OK;
 }
 

@@ -3,6 +3,7 @@
 
 #include <cuda_runtime.h>
 
+#include <atomic>
 #include <cstddef>
 #include <cstdint>
 #include <map>
@@ -94,6 +95,7 @@ struct wd_ctx {
     // launch-shape cache filled by the autotuner: problem key -> (threads, variant)
     std::mutex tune_mu;
     std::map<std::string, std::pair<int, int>> tuned;
+    std::atomic<bool> any_tuned{false};   // set with the first entry: until then no launch looks for its own
     std::string tune_file;   // on-disk cache (WD_TUNE_CACHE), empty if none
 };
 
