@@ -25,21 +25,60 @@ std::string hop_key(const wd_ctx *ctx, const HopArgs &A, int prec, int recon, in
     return buf;
 }
 
-// Untuned defaults, from tuning runs on GB300 (32^4, 24^3x48, 16^3x32): the
-// FP32/FP16/BF16 kernels are fastest with 64-thread blocks and memory
-// schedule 1; even-odd hops (each link read once) load the links without L1
-// allocation, FP32 ones with schedule 0 (24^3x48: 40.1 against 43.3 us for
-// schedule 1; 32^4: 62.6 against 63.8 us) and the 16-bit ones with the
-// spin-paired kernel (schedule 0); FP64 (bound by the FP64 pipe) with three
-// threads per site (128: the block size of an open-boundary pass, which uses
-// hop_kernel).
-static std::pair<int, int> hop_default(int prec, int nrhs, int nparity)
+// Default shape of the shared-link kernel: {threads, variant}.
+// Threads: 4 warps per block, or 3 where that leaves fewer of them idle in the last
+// pass over the fields (large grids; us, 128 / 96 threads: 32^4 even-odd, FP32, 5
+// fields 186.6 / 177.9, 6 fields 207.0 / 197.2, 7 FP16 fields on 24^3 x 48 118.3 /
+// 120.9; small grids want the warps: 12 x 14 x 10 x 18, 5 fields 11.6 / 12.9).
+// Site order: a source spinor is read as t+ neighbour and again, 2 Lz slices
+// later, as t- neighbour.  Where what is touched in between exceeds about half of L2 the
+// slices are visited in the widest z-strips whose 2 w slices take no more than 0.4
+// of it.  us, natural order / strips of 16 / of 8 (MB between the two reads in
+// natural order; L2 129 MB): FP32 full on 32^4, 12 fields 855 / 772 / 734 (170), 6
+// fields 422 / 403 / 408 (94), 4 fields 300 / 300 / 310 (69); even-odd, 12 fields 370 /
+// 357 / 359 (94), 5 fields 185 / 195 / 197 (50); FP16 even-odd, 12 fields 275 / 284 / 286 (50).
+static std::pair<int, int> mrhs_default(const HopArgs &A, int prec, int recon, int nrhs)
 {
+    const long long blocks = (long long)((A.vh + 31) / 32) * A.nparity;
+    int threads = 128, variant = HOP_MRHS_VARIANT;
+    if (prec == WD_F64) return {threads, variant};   // bound by the FP64 pipe
+    if (!mrhs_small(blocks, threads) && 3 * ((nrhs + 2) / 3) < 4 * ((nrhs + 3) / 4)) threads = 96;
+    const double field = half_field_bytes(1, prec), link = link_block_bytes(1, link_prec(prec), recon);
+    const double slice = (double)(A.L[0] / 2) * A.L[1] * A.nparity * (2 * nrhs * field + 8 / A.nparity * link);
+    const double l2 = (double)device_l2_bytes();
+    if (2 * A.L[2] * slice > 0.55 * l2) {
+        for (int v = 5; v <= 7; ++v)   // strips of 16, 8, 4
+            if (hop_mrhs_strip(v) < A.L[2] && (2 * hop_mrhs_strip(v) * slice <= 0.4 * l2 || v == 7)) {
+                variant = v;
+                break;
+            }
+    }
+    return {threads, variant};
+}
+
+// Untuned defaults, from tuning runs on GB300 (8^4 to 32^4): 64-thread blocks;
+// full operator: schedule 1, with 16-bit storage and 12-real links schedule 2 on
+// large lattices (us, schedule 1 / 2: 24^3 x 48 43.9 / 41.5, 32^4 66.1 / 62.2, 16^3 x 32 9.2 /
+// 9.5); even-odd hops (each link read once) load the links without L1 allocation,
+// FP32 ones with schedule 0 (24^3 x 48: 42.2 against 43.4 us for schedule 1), with the
+// axpy term and 18-real links on large lattices schedule 1 (24^3 x 48 47.3 / 45.1,
+// 32^4 70.0 / 67.4), and the 16-bit ones with the spin-paired kernel (schedule 0); FP64
+// (bound by the FP64 pipe) with three threads per site (128: the block size of an
+// open-boundary pass, which uses hop_kernel).
+constexpr int HOP_LARGE = 300000;   // sites of one parity: 24^3 x 48 has 331,776, 16^3 x 32 65,536
+
+static std::pair<int, int> hop_default(const HopArgs &A, int prec, int recon, int nrhs)
+{
+    const bool large = A.vh >= HOP_LARGE, hx = A.x[0] != nullptr || A.x[1] != nullptr;
     if (prec == WD_DF) return {96, HOP_ROW_VARIANT};   // double-word: three threads per site
-    if (nrhs > 1) return {128, HOP_MRHS_VARIANT};   // shared-link kernel, 4 fields at a time
+    if (nrhs > 1) return mrhs_default(A, prec, recon, nrhs);
     if (prec == WD_F64) return {128, HOP_ROW_VARIANT};
-    if (nparity == 1 && (prec == WD_F16 || prec == WD_BF16)) return {64, HOP_SP0_VARIANT};
-    return {64, nparity == 1 ? HOP_NA0_VARIANT : 1};
+    if (prec == WD_F32) {
+        if (A.nparity == 2) return {64, 1};
+        return {64, large && hx && recon == 18 ? HOP_NA1_VARIANT : HOP_NA0_VARIANT};
+    }
+    if (A.nparity == 1) return {64, HOP_SP0_VARIANT};
+    return {64, large && recon == 12 ? 2 : 1};
 }
 
 int hop_launch_cfg(const HopArgs &A, int prec, int recon, int dagger, int nrhs, int threads, int variant,
@@ -62,7 +101,7 @@ int hop_launch_cfg(const HopArgs &A, int prec, int recon, int dagger, int nrhs, 
 int hop_launch(wd_ctx *ctx, const HopArgs &A, int prec, int recon, int dagger, int nrhs, cudaStream_t s)
 {
     // the key of a launch is a string: 1 us to build, on a call of 3 us
-    auto cfg = hop_default(prec, nrhs, A.nparity);
+    auto cfg = hop_default(A, prec, recon, nrhs);
     if (ctx->any_tuned.load(std::memory_order_acquire)) cfg = tuned_config(ctx, hop_key(ctx, A, prec, recon, nrhs), cfg);
     return hop_launch_cfg(A, prec, recon, dagger, nrhs, cfg.first, cfg.second, s);
 }

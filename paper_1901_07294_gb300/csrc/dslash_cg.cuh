@@ -144,8 +144,8 @@ template <int P> struct CgResidStore {
 };
 
 // One hop of the iteration with its share of the vector work: the kernel of the
-// untuned even-odd hops (schedule 0, links without L1 allocation; 16-bit
-// storage: spin-paired).
+// untuned even-odd hops (links without L1 allocation; FP32: schedule 1 with the
+// axpy term, else 0; 16-bit storage: spin-paired, schedule 0).
 template <int P, int RECON, int STEP>
 __global__ void __launch_bounds__(256, 2) hop_cg_kernel(const HopArgs A, const CgHop C, const int nparts)
 {
@@ -167,7 +167,7 @@ __global__ void __launch_bounds__(256, 2) hop_cg_kernel(const HopArgs A, const C
     constexpr bool DAG = STEP != CG_NORM, HX = STEP != CG_ALPHA;
     auto run = [&](const auto &epi) {
         if constexpr (Prec<P>::scaled) sp_site<P, RECON, DAG, HX, 0, true>(A, A.parity0, i, 0, epi);
-        else hop_site<P, RECON, DAG, HX, 0, false, true>(A, A.parity0, i, 0, epi);
+        else hop_site<P, RECON, DAG, HX, HX ? 1 : 0, false, true>(A, A.parity0, i, 0, epi);
     };
     if constexpr (STEP == CG_NORM) run(CgNormStore<P>{C.site});
     else if constexpr (STEP == CG_ALPHA) run(HopStore<P, false>{});

@@ -99,22 +99,25 @@ cudaError_t wd_launch(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t sm
     return e;
 }
 
-// SMs of the current device (queried once per device).
-inline int device_sm_count()
+// An attribute of the current device (queried once per device), `def` if it
+// cannot be read.
+template <cudaDeviceAttr ATTR> inline int device_attr(int def)
 {
     static std::atomic<int> cache[64] = {};
     int dev = -1;
-    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 152;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return def;
     int v = cache[dev].load(std::memory_order_relaxed);
     if (v == 0) {
-        if (cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || v <= 0) {
+        if (cudaDeviceGetAttribute(&v, ATTR, dev) != cudaSuccess || v <= 0) {
             cudaGetLastError();
-            v = 152;
+            v = def;
         }
         cache[dev].store(v, std::memory_order_relaxed);
     }
     return v;
 }
+inline int device_sm_count() { return device_attr<cudaDevAttrMultiProcessorCount>(152); }
+inline int device_l2_bytes() { return device_attr<cudaDevAttrL2CacheSize>(129 << 20); }
 
 // Dynamic shared memory that keeps a grid of less than a full wave evenly
 // spread.  A kernel dispatched while its predecessor's last blocks run finds
