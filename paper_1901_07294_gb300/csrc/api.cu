@@ -314,7 +314,7 @@ int ctx_workspace(wd_ctx *ctx, size_t bytes, char **out)
             ctx->d_work = nullptr;
             ctx->work_bytes = 0;
         }
-        if (cudaMalloc(&ctx->d_work, bytes) != cudaSuccess) {
+        if (dev_malloc(ctx, &ctx->d_work, bytes) != cudaSuccess) {
             cudaGetLastError();
             return set_error(WD_ENOMEM, "cudaMalloc of %zu bytes of solver workspace failed", bytes);
         }
@@ -333,7 +333,7 @@ int ctx_aux_workspace(wd_ctx *ctx, size_t bytes, char **out)
             ctx->d_aux = nullptr;
             ctx->aux_bytes = 0;
         }
-        if (cudaMalloc(&ctx->d_aux, bytes) != cudaSuccess) {
+        if (dev_malloc(ctx, &ctx->d_aux, bytes) != cudaSuccess) {
             cudaGetLastError();
             return set_error(WD_ENOMEM, "cudaMalloc of %zu bytes of solver workspace failed", bytes);
         }
@@ -341,6 +341,81 @@ int ctx_aux_workspace(wd_ctx *ctx, size_t bytes, char **out)
     }
     *out = ctx->d_aux;
     return WD_OK;
+}
+
+void SolvePool::free_entry(const Entry &e)
+{
+    if (e.s) {
+        cudaStreamSynchronize(e.s);
+        cudaStreamDestroy(e.s);
+    }
+    if (e.mem) cudaFree(e.mem);
+    if (e.h) cudaFreeHost(e.h);
+}
+
+bool SolvePool::take(size_t bytes, Entry &e)
+{
+    std::lock_guard<std::mutex> lk(mu);
+    for (size_t k = idle.size(); k-- > 0;)
+        if (idle[k].bytes == bytes) {
+            e = idle[k];
+            held -= bytes;
+            idle.erase(idle.begin() + (long)k);
+            return true;
+        }
+    return false;
+}
+
+// Takes the oldest entry out.
+bool SolvePool::pop_oldest(Entry &e)
+{
+    if (idle.empty()) return false;
+    e = idle.front();
+    held -= e.bytes;
+    idle.erase(idle.begin());
+    return true;
+}
+
+void SolvePool::put(const Entry &e)
+{
+    for (;;) {
+        Entry old;   // freed after the lock is dropped: the oldest make room
+        {
+            std::lock_guard<std::mutex> lk(mu);
+            if (closed || e.bytes > MAX_BYTES) {
+                old = e;
+            } else if (idle.size() < MAX_ENTRIES && held + e.bytes <= MAX_BYTES) {
+                idle.push_back(e);   // within the reserved capacity: does not allocate
+                held += e.bytes;
+                return;
+            } else {
+                pop_oldest(old);
+            }
+        }
+        free_entry(old);
+        if (old.mem == e.mem) return;
+    }
+}
+
+void SolvePool::trim()
+{
+    for (;;) {
+        Entry old;
+        {
+            std::lock_guard<std::mutex> lk(mu);
+            if (!pop_oldest(old)) return;
+        }
+        free_entry(old);
+    }
+}
+
+void SolvePool::close()
+{
+    {
+        std::lock_guard<std::mutex> lk(mu);
+        closed = true;
+    }
+    trim();
 }
 
 int gauge_layout(const wd_gauge *gc, int prec, int recon, const char **out)
@@ -359,7 +434,7 @@ int gauge_layout(const wd_gauge *gc, int prec, int recon, const char **out)
     DeviceGuard dg(g->device);
     const size_t blk = link_block_bytes(g->geo.Vh, prec, recon);
     char *buf = nullptr;
-    if (cudaMalloc(&buf, 8 * blk) != cudaSuccess) {
+    if (dev_malloc(g->ctx, &buf, 8 * blk) != cudaSuccess) {
         cudaGetLastError();
         return set_error(WD_ENOMEM, "cudaMalloc of %zu bytes for a gauge layout failed", 8 * blk);
     }
@@ -416,8 +491,12 @@ int wd_ctx_create(int device, wd_ctx **out)
     int n = 0;
     WD_CUDA_TRY(cudaGetDeviceCount(&n));
     if (device < 0 || device >= n) return set_error(WD_EINVAL, "device %d out of range (%d devices)", device, n);
-    wd_ctx *c = new (std::nothrow) wd_ctx();
-    if (!c) return set_error(WD_ENOMEM, "host allocation failed");
+    wd_ctx *c = nullptr;
+    try {
+        c = new wd_ctx();
+    } catch (...) {
+        return set_error(WD_ENOMEM, "host allocation failed");
+    }
     c->device = device;
     cudaDeviceProp prop;
     cudaError_t e = cudaGetDeviceProperties(&prop, device);
@@ -451,6 +530,7 @@ int wd_ctx_destroy(wd_ctx *ctx)
     if (!ctx) return WD_OK;
     {
         DeviceGuard dg(ctx->device);
+        ctx->solve_pool->close();
         cudaFree(ctx->d_partials);
         cudaFree(ctx->d_ticket);
         cudaFree(ctx->d_scal);
@@ -637,7 +717,7 @@ int wd_gauge_create(wd_ctx *ctx, const int dims[4], const double *links, int lin
     g->device = ctx->device;
     g->geo = geo;
     const size_t nb = (size_t)geo.V * 4 * 18 * sizeof(double);
-    if (cudaMalloc(&g->canonical, nb) != cudaSuccess) {
+    if (dev_malloc(ctx, &g->canonical, nb) != cudaSuccess) {
         cudaGetLastError();
         delete g;
         return set_error(WD_ENOMEM, "cudaMalloc of %zu bytes for the gauge field failed", nb);

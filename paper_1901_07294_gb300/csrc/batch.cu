@@ -445,7 +445,7 @@ int run_persistent(wd_ctx *ctx, int n, const wd_solve_desc *d, wd_cg_stats *stat
                      (size_t)((vh + 255) / 256) * 8 * 2 * 2 * sizeof(double) + 256;
         }
         DevBuf work, meta;
-        if (cudaMalloc(&work.p, bytes) != cudaSuccess) {
+        if (dev_malloc(ctx, &work.p, bytes) != cudaSuccess) {
             cudaGetLastError();
             return set_error(WD_ENOMEM, "cudaMalloc of %zu bytes for the persistent batch failed", bytes);
         }

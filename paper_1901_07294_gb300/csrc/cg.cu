@@ -238,7 +238,7 @@ int cg_run_graph(wd_ctx *ctx, const wd_gauge *g, double mass, char *x, const cha
         if (rc == WD_OK && cudaStreamSynchronize(q.s) != cudaSuccess) rc = set_error(WD_ECUDA, "graph replay failed");
         if (rc == WD_OK) rc = gs_after(ctx, q);
     }
-    gs_release(q);
+    gs_release(q, rc == WD_ECUDA ? nullptr : ctx->solve_pool.get());
     st.iters = q.iters;
     st.reliable_updates = q.updates;
     st.true_rel_resid = q.rel;

@@ -375,7 +375,7 @@ int wd_dd_create(wd_ctx *ctx, const int dims[4], int nsub, const double *links, 
         d->sub.push_back(g);
     }
     d->slot = 2 * face_bytes(WD_F64, d->nf);
-    if (cudaMalloc(&d->buf, (size_t)2 * nsub * 2 * d->slot) != cudaSuccess ||
+    if (dev_malloc(ctx, &d->buf, (size_t)2 * nsub * 2 * d->slot) != cudaSuccess ||
         cudaStreamCreateWithFlags(&d->side, cudaStreamNonBlocking) != cudaSuccess ||
         cudaEventCreateWithFlags(&d->ev_in, cudaEventDisableTiming) != cudaSuccess ||
         cudaEventCreateWithFlags(&d->ev_halo, cudaEventDisableTiming) != cudaSuccess) {

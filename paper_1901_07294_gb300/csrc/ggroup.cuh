@@ -297,8 +297,8 @@ template <int PS> int build(const wd_ctx *ctx, GGroup &g)
 inline int gg_create(const wd_ctx *ctx, GGroup &g)
 {
     WD_CUDA_TRY(cudaStreamCreateWithFlags(&g.s, cudaStreamNonBlocking));
-    if (cudaMalloc(&g.d_table, sizeof(GTable)) != cudaSuccess ||
-        cudaMalloc(&g.d_hs, sizeof(double) * GG_MAX * GS_NSCAL) != cudaSuccess) {
+    if (dev_malloc(ctx, &g.d_table, sizeof(GTable)) != cudaSuccess ||
+        dev_malloc(ctx, &g.d_hs, sizeof(double) * GG_MAX * GS_NSCAL) != cudaSuccess) {
         cudaGetLastError();
         return set_error(WD_ENOMEM, "allocation of a request group's tables failed");
     }

@@ -231,14 +231,22 @@ template <int PS> int init(const wd_ctx *ctx, GSolve &q, bool with_graph)
     default: { constexpr int PS = PREC_F32; return CALL; }                    \
     }
 
-// Allocates a solve's device workspace, pinned scalars and stream.  Returns
-// WD_ENOMEM if the workspace does not fit.
-inline int gs_alloc(GSolve &q)
+// A solve's device workspace, pinned scalars and stream: idle ones of the same
+// size from the context's pool, else new ones.  Returns WD_ENOMEM if the
+// workspace does not fit.
+inline int gs_alloc(const wd_ctx *ctx, GSolve &q)
 {
     q.vh = q.gauge->geo.Vh;
     q.prec = q.opts.inner_prec;
     const size_t bytes = gs_footprint(q.vh, q.prec);
-    if (cudaMalloc(&q.mem, bytes) != cudaSuccess) {
+    SolvePool::Entry e;
+    if (ctx->solve_pool->take(bytes, e)) {
+        q.mem = e.mem;
+        q.h = e.h;
+        q.s = e.s;
+        return WD_OK;
+    }
+    if (dev_malloc(ctx, &q.mem, bytes) != cudaSuccess) {
         cudaGetLastError();
         q.mem = nullptr;
         return set_error(WD_ENOMEM, "cudaMalloc of %zu bytes of solve workspace failed", bytes);
@@ -280,7 +288,7 @@ inline int gs_bind(const wd_ctx *ctx, GSolve &q, bool graph = true)
 // gs_alloc + gs_bind.
 inline int gs_setup(const wd_ctx *ctx, GSolve &q)
 {
-    WD_TRY(gs_alloc(q));
+    WD_TRY(gs_alloc(ctx, q));
     return gs_bind(ctx, q);
 }
 
@@ -435,13 +443,15 @@ inline void gs_release_graph(GSolve &q)
     q.exec = nullptr;
 }
 
-inline void gs_release(GSolve &q)
+// Gives a solve's resources back: to `pool`, or (no pool, work that failed, or an
+// incomplete set) to the device.
+inline void gs_release(GSolve &q, SolvePool *pool = nullptr)
 {
-    if (q.s) cudaStreamSynchronize(q.s);
+    const bool idle = !q.s || cudaStreamSynchronize(q.s) == cudaSuccess;
     if (q.exec) cudaGraphExecDestroy(q.exec);
-    if (q.s) cudaStreamDestroy(q.s);
-    if (q.mem) cudaFree(q.mem);
-    if (q.h) cudaFreeHost(q.h);
+    const SolvePool::Entry e{q.mem ? gs_footprint(q.vh, q.prec) : 0, q.mem, q.h, q.s};
+    if (pool && idle && e.mem && e.h && e.s) pool->put(e);
+    else SolvePool::free_entry(e);
     q.exec = nullptr;
     q.s = nullptr;
     q.mem = nullptr;

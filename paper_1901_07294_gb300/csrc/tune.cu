@@ -71,8 +71,8 @@ int wd_tune_dslash(wd_ctx *ctx, const wd_gauge *g, int prec, int recon, int full
     const size_t half = half_field_bytes(A.vh, prec);
     const size_t field = (full ? 2 : 1) * half * (size_t)nrhs;
     char *in = nullptr, *out = nullptr, *x = nullptr;
-    if (cudaMalloc(&in, field) != cudaSuccess || cudaMalloc(&out, field) != cudaSuccess ||
-        (!full && with_x && cudaMalloc(&x, field) != cudaSuccess)) {
+    if (dev_malloc(ctx, &in, field) != cudaSuccess || dev_malloc(ctx, &out, field) != cudaSuccess ||
+        (!full && with_x && dev_malloc(ctx, &x, field) != cudaSuccess)) {
         cudaGetLastError();
         cudaFree(in);
         cudaFree(out);

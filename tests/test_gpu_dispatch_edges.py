@@ -98,3 +98,32 @@ def test_full_pack_tiles_equal_half_packs(ctx, dims, prec):
     wd.unpack(ctx, dims, wd.SITES_ODD, prec, halves[half:], two)
     assert torch.equal(one, two)
     assert rel_max_err(one.cpu().numpy()[parity(dims).repeat(24) == 0], psi.view(-1).cpu().numpy()[parity(dims).repeat(24) == 0]) < 2.0 ** -8
+
+
+def test_kept_workspaces_give_the_same_bits():
+    """A solve in a workspace that another solve has used, and one queued after it, equal the first;
+    closing a queue after its context is allowed."""
+    import torch
+    ctx = wd.Context(0)
+    dims, other = (8, 8, 8, 8), (4, 6, 8, 10)
+    g, h = (wd.Gauge(ctx, d, synth.gauge(d, seed=95)) for d in (dims, other))
+    b, c = (pack_field(ctx, d, wd.SITES_EVEN, wd.F64, synth.even_spinor(d, seed=96)) for d in (dims, other))
+    xs = []
+    for _ in range(3):
+        x, y = torch.zeros_like(b), torch.zeros_like(c)
+        wd.cg_solve(ctx, g, 0.2, x, b, tol=1e-10, inner_prec=wd.F16, use_graph=True)
+        wd.cg_solve(ctx, h, 0.3, y, c, tol=1e-9, inner_prec=wd.F16, use_graph=True)
+        xs.append((x, y))
+    assert all(torch.equal(u, v) for p in xs[1:] for u, v in zip(xs[0], p))
+    batches = []
+    for _ in range(2):
+        out = [torch.zeros_like(b) for _ in range(3)]
+        wd.cg_solve_batch(ctx, [dict(gauge=g, mass=0.1 + 0.1 * k, tol=1e-10, x=v, b=b, inner_prec=wd.F16)
+                                for k, v in enumerate(out)], mode=wd.BATCH_GRAPH)
+        batches.append(out)
+    assert all(torch.equal(u, v) for u, v in zip(*batches))
+    q = wd.Queue(ctx, 1 << 30, 2)
+    x = torch.zeros_like(b)
+    q.wait(q.submit(dict(gauge=g, mass=0.2, tol=1e-10, x=x, b=b, inner_prec=wd.F16)))
+    ctx.close()
+    q.close()
