@@ -72,8 +72,9 @@ int wd_axpby(wd_ctx *ctx, const int dims[4], int sites, int prec, double a, cons
     const int n = blas_sites(dims, sites, g);
     if (n < 0) return n;
     WD_PREC_SWITCH(prec, {
-        OpAxpby<P, P> op{field_ref<P>(x, g.Vh), field_ref<P>(y, g.Vh), a, b};
-        return run_blas(ctx, op, n, (cudaStream_t)stream);
+        const auto fx = field_ref<P>(x, g.Vh), fy = field_ref<P>(y, g.Vh);
+        if (P == PREC_F64 && b == 1.0) return run_blas(ctx, OpAxpby<P, P, P == PREC_F64>{fx, fy, a, b}, n, (cudaStream_t)stream);
+        return run_blas(ctx, OpAxpby<P, P>{fx, fy, a, b}, n, (cudaStream_t)stream);
     });
     return WD_OK;
 }

@@ -56,6 +56,10 @@ template <typename Op> inline int blas_resident_blocks()
 // reduction order is too.
 template <typename Op> inline int blas_grid_for(const wd_ctx *ctx, int nsite)
 {
+    if constexpr (flat_vectors<Op> > 0) {   // one vector per thread up to the cap
+        const long long n = (long long)nsite * flat_vectors<Op>;
+        nsite = n < (1 << 30) ? (int)n : (1 << 30);
+    }
     if constexpr (Op::NR == 0) return blas_grid(ctx, nsite);
     const int want = (nsite + BLAS_THREADS - 1) / BLAS_THREADS;
     const int fit = blas_resident_blocks<Op>();

@@ -153,7 +153,7 @@ int cg_run(wd_ctx *ctx, const wd_gauge *g, double mass, char *x, const char *b, 
         if (update) {
             // x += x_lo (FP64), then the true residual with the FP64 operator
             if constexpr (PS == PREC_F64) {
-                WD_TRY(run_blas(ctx, OpAxpby<PX, PREC_F64>{FX(xs), F64(x), 1.0, 1.0}, vh, s));
+                WD_TRY(run_blas(ctx, OpAxpby<PX, PREC_F64, true>{FX(xs), F64(x), 1.0, 1.0}, vh, s));
                 WD_CUDA_TRY(cudaMemsetAsync(xs, 0, hx, s));
             } else {
                 WD_TRY(run_blas(ctx, OpFlushX<PX, PS>{F64(x), FX(xs), FS(ps), d + 2}, vh, s));
@@ -204,7 +204,7 @@ int cg_run(wd_ctx *ctx, const wd_gauge *g, double mass, char *x, const char *b, 
         r2 = r2_new;
     }
     if (!converged && status == WD_OK) {
-        WD_TRY(run_blas(ctx, OpAxpby<PX, PREC_F64>{FX(xs), F64(x), 1.0, 1.0}, vh, s));
+        WD_TRY(run_blas(ctx, OpAxpby<PX, PREC_F64, true>{FX(xs), F64(x), 1.0, 1.0}, vh, s));
         WD_TRY(true_residual(WD_F64, vh, x, b, r, ax, d + 4, mdagm_outer, blas));
         WD_TRY(read_scalars(ctx, 4, 1, s));
         r2_true = h[4];

@@ -137,7 +137,7 @@ int bicg_run(wd_ctx *ctx, const wd_gauge *g, double mass, char *x, const char *b
         else update = update || r2 <= std::fmax(stop2, delta * delta * r2_restart);
         if (!update) continue;
         // x += x_lo (FP64), then the true residual with the FP64 operator
-        WD_TRY(run_blas(ctx, OpAxpby<PX, PREC_F64>{FX(xs), F64(x), 1.0, 1.0}, vh, s));
+        WD_TRY(run_blas(ctx, OpAxpby<PX, PREC_F64, true>{FX(xs), F64(x), 1.0, 1.0}, vh, s));
         WD_CUDA_TRY(cudaMemsetAsync(xs, 0, hx, s));
         // an update that the iterated residual's convergence triggered is a
         // convergence check: FP64 directly, as are all updates after a failed check
@@ -175,7 +175,7 @@ int bicg_run(wd_ctx *ctx, const wd_gauge *g, double mass, char *x, const char *b
         }
     }
     if (!converged && status == WD_OK) {
-        WD_TRY(run_blas(ctx, OpAxpby<PX, PREC_F64>{FX(xs), F64(x), 1.0, 1.0}, vh, s));
+        WD_TRY(run_blas(ctx, OpAxpby<PX, PREC_F64, true>{FX(xs), F64(x), 1.0, 1.0}, vh, s));
         WD_TRY(true_residual(WD_F64, vh, x, b, r, ax, d + 4, mhat_outer, blas));
         WD_TRY(read_scal(ctx, 4, 1, s));
         r2_true = h[4];
@@ -263,7 +263,7 @@ int cgne_schur(wd_ctx *ctx, const wd_gauge *g, double mass, char *x_e, const cha
         st.iters += cs.iters;
         st.reliable_updates += cs.reliable_updates;
         if (rc != WD_OK && rc != WD_ENOCONV) return rc;
-        WD_TRY(run_blas(ctx, OpAxpby<PREC_F64, PREC_F64>{F64(e), F64(x_e), 1.0, 1.0}, vh, s));
+        WD_TRY(run_blas(ctx, OpAxpby<PREC_F64, PREC_F64, true>{F64(e), F64(x_e), 1.0, 1.0}, vh, s));
         WD_TRY(apply_mhat(g, WD_F64, o.outer_recon, mass, x_e, c, t_o, 0, s));
         WD_TRY(run_blas(ctx, OpXmyNorm<PREC_F64>{F64(bh), F64(c), F64(rh), d + 4}, vh, s));
         WD_TRY(read_scal(ctx, 4, 1, s));
