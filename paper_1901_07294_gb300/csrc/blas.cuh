@@ -258,19 +258,18 @@ template <int PX, int PR> struct OpCgUpdate {
     __device__ __forceinline__ void finish(const double (&s)[1]) const { out[0] = s[0]; }
 };
 
-// r = b - y; returns |r|^2 (used for the true residual, FP64; y may be a
-// double-word field, widened exactly to FP64 first).
-template <int P, int PY = P> struct OpXmyNorm {
+// r = b - y; returns |r|^2 (the full solve's residuals, FP64).
+template <int P> struct OpXmyNorm {
     static constexpr int NR = 1;
     FieldRef<P> b;
-    FieldRef<PY> y;
+    FieldRef<P> y;
     FieldRef<P> r;
     double *out;
     __device__ __forceinline__ void site(int j, double (&acc)[1]) const
     {
         using T = typename Prec<P>::real;
         T bv[24];
-        typename Prec<PY>::real yv[24];
+        typename Prec<P>::real yv[24];
         b.load(j, bv);
         y.load(j, yv);
         T s = 0;
@@ -281,6 +280,44 @@ template <int P, int PY = P> struct OpXmyNorm {
         }
         r.store(j, bv);
         acc[0] += to_real<double>(s);
+    }
+    __device__ __forceinline__ void finish(const double (&s)[1]) const { out[0] = s[0]; }
+};
+
+// r = b - y in FP64 (y may be a double-word field, widened exactly), |r|^2 from the
+// FP64 values, r stored in the precision PS of the iteration it restarts.  One pass
+// where storing r in FP64 and converting it took two: 58 + 17 -> 62 us on 24^3 x 48
+// (double-word y, FP16 r).  Bound by the FP64 pipe (three instructions per real: 38
+// us); with the conversion to FP32 on that pipe too it took 74 us (FP64 y: 55 ->
+// 43 us).  The whole FP16 CG there: 19.78 -> 19.62 ms.
+template <int PY, int PS> struct OpResidual {
+    static constexpr int NR = 1;
+    FieldRef<PREC_F64> b;
+    FieldRef<PY> y;
+    FieldRef<PS> r;
+    double *out;
+    __device__ __forceinline__ void site(int j, double (&acc)[1]) const
+    {
+        typename Prec<PS>::real v[24];
+        double s = 0;
+        const int h = j >= b.vh, i = j - h * b.vh;
+#pragma unroll
+        for (int k = 0; k < 12; ++k) {   // planes of two reals, the same in both formats
+            const size_t o = h * b.half_bytes + ((size_t)k * b.vh + i) * 16;
+            double d[2];
+            typename Prec<PY>::real yv[2];
+            unpack16<PREC_F64>(ldg16(b.p + o), d, 1.0f);
+            unpack16<PY>(ldg16(y.p + o), yv, 1.0f);
+#pragma unroll
+            for (int l = 0; l < 2; ++l) {
+                d[l] -= to_real<double>(yv[l]);
+                s = fma(d[l], d[l], s);
+                if constexpr (PS == PREC_F64) v[2 * k + l] = d[l];
+                else v[2 * k + l] = f64_to_f32(d[l]);
+            }
+        }
+        r.store(j, v);
+        acc[0] += s;
     }
     __device__ __forceinline__ void finish(const double (&s)[1]) const { out[0] = s[0]; }
 };
@@ -318,29 +355,43 @@ template <int PX, int P> struct OpXp {
 };
 
 // x += x_lo + alpha p for the FP64 solution x, and x_lo = 0: the start of a
-// reliable update, with the step of the last iteration (not yet in x_lo)
-template <int PX, int P> struct OpFlushX {
+// reliable update, with the step of the last iteration (not yet in x_lo).  DFX: the
+// new x in double-word form too, for the update's operator: that copy as a pass of
+// its own reads x again and takes 29 us on 24^3 x 48, this whole one 59 us (820
+// bytes per site, 4.6 TB/s).
+template <int PX, int P, bool DFX> struct OpFlushX {
     static constexpr int NR = 0;
     FieldRef<PREC_F64> x;
     FieldRef<PX> xlo;
     FieldRef<P> p;
+    FieldRef<PREC_DF> xd;
     const double *alpha;
     __device__ __forceinline__ void site(int j, double (&)[1]) const
     {
         using TX = typename Prec<PX>::real;
         const TX al = (TX)*alpha;
-        double xv[24];
         TX lo[24];
         typename Prec<P>::real pv[24];
         xlo.load(j, lo);
         p.load(j, pv);
-        x.load(j, xv);
 #pragma unroll
-        for (int k = 0; k < 24; ++k) {
-            xv[k] += to_real<double>(fma(al, to_real<TX>(pv[k]), lo[k]));
-            lo[k] = TX(0);
+        for (int k = 0; k < 24; ++k) lo[k] = fma(al, to_real<TX>(pv[k]), lo[k]);
+        const int h = j >= x.vh, i = j - h * x.vh;
+#pragma unroll
+        for (int k = 0; k < 12; ++k) {   // planes of two reals, the same in both formats
+            const size_t o = h * x.half_bytes + ((size_t)k * x.vh + i) * 16;
+            double v[2];
+            unpack16<PREC_F64>(ldg16(x.p + o), v, 1.0f);
+            v[0] += to_real<double>(lo[2 * k]);
+            v[1] += to_real<double>(lo[2 * k + 1]);
+            stg16(x.p + o, pack16<PREC_F64>(v, 1.0f));
+            if constexpr (DFX) {
+                const df d[2] = {to_real<df>(v[0]), to_real<df>(v[1])};
+                stg16(xd.p + o, pack16<PREC_DF>(d, 1.0f));
+            }
         }
-        x.store(j, xv);
+#pragma unroll
+        for (int k = 0; k < 24; ++k) lo[k] = TX(0);
         xlo.store(j, lo);
     }
     __device__ __forceinline__ void finish(const double (&)[1]) const {}

@@ -85,23 +85,25 @@ inline int outer_prec_of(const wd_cg_opts &o)
     return (o.inner_prec != WD_F64 && o.outer_prec == WD_DF) ? WD_DF : WD_F64;
 }
 
-// r = b - A x and |r|^2 -> *out for FP64 even half fields x, b, r; ax is
-// scratch for A x.  apply(prec, in, out) applies A in precision prec;
+// rs = b - A x (in the iteration's precision PS) and its |b - A x|^2 -> *out for FP64
+// even half fields x, b; ax is scratch for A x, xd for x in double-word form
+// (x_ready: already there).  apply(prec, in, out) applies A in precision prec;
 // blas(op) launches a BLAS operation on the caller's stream and scratch.  In
-// double-word arithmetic x is first converted into r's buffer (r is written
-// only by the last step), and A x is widened exactly to FP64 in the difference.
-template <typename Apply, typename Blas>
-int true_residual(int op, int vh, const char *x, const char *b, char *r, char *ax, double *out, Apply &&apply,
-                  Blas &&blas)
+// double-word arithmetic A x is widened exactly to FP64 in the difference.
+template <int PS, typename Apply, typename Blas>
+int true_residual(int op, int vh, const char *x, const char *b, char *rs, char *xd, bool x_ready, char *ax,
+                  double *out, Apply &&apply, Blas &&blas)
 {
-    const FieldRef<PREC_F64> fb = field_ref<PREC_F64>(b, vh), fr = field_ref<PREC_F64>(r, vh);
+    const FieldRef<PREC_F64> fb = field_ref<PREC_F64>(b, vh);
+    const FieldRef<PS> fr = field_ref<PS>(rs, vh);
     if (op == WD_DF) {
-        WD_TRY(blas(OpConvert<PREC_DF, PREC_F64>{field_ref<PREC_DF>(r, vh), field_ref<PREC_F64>(x, vh)}));
-        WD_TRY(apply(WD_DF, (const char *)r, ax));
-        return blas(OpXmyNorm<PREC_F64, PREC_DF>{fb, field_ref<PREC_DF>(ax, vh), fr, out});
+        if (!x_ready)
+            WD_TRY(blas(OpConvert<PREC_DF, PREC_F64>{field_ref<PREC_DF>(xd, vh), field_ref<PREC_F64>(x, vh)}));
+        WD_TRY(apply(WD_DF, (const char *)xd, ax));
+        return blas(OpResidual<PREC_DF, PS>{fb, field_ref<PREC_DF>(ax, vh), fr, out});
     }
     WD_TRY(apply(WD_F64, x, ax));
-    return blas(OpXmyNorm<PREC_F64>{fb, field_ref<PREC_F64>(ax, vh), fr, out});
+    return blas(OpResidual<PREC_F64, PS>{fb, field_ref<PREC_F64>(ax, vh), fr, out});
 }
 
 } // namespace wd

@@ -108,8 +108,7 @@ int cg_run(wd_ctx *ctx, const wd_gauge *g, double mass, char *x, const char *b, 
         WD_CUDA_TRY(cudaStreamSynchronize(s));
         return std::isfinite(b2) ? WD_OK : set_error(WD_EINVAL, "source is not finite");
     }
-    WD_CUDA_TRY(cudaMemcpyAsync(r, b, h64, cudaMemcpyDeviceToDevice, s));
-    WD_TRY(run_blas(ctx, OpConvert<PS, PREC_F64>{FS(rs), F64(r)}, vh, s));
+    WD_TRY(run_blas(ctx, OpConvert<PS, PREC_F64>{FS(rs), F64(b)}, vh, s));
     WD_CUDA_TRY(cudaMemcpyAsync(ps, rs, hs, cudaMemcpyDeviceToDevice, s));
     WD_CUDA_TRY(cudaMemsetAsync(xs, 0, hx, s));
 
@@ -152,23 +151,25 @@ int cg_run(wd_ctx *ctx, const wd_gauge *g, double mass, char *x, const char *b, 
         else update = r2_new <= std::fmax(stop2, delta * delta * r2_restart);
         if (update) {
             // x += x_lo (FP64), then the true residual with the FP64 operator
-            if constexpr (PS == PREC_F64) {
-                WD_TRY(run_blas(ctx, OpAxpby<PX, PREC_F64, true>{FX(xs), F64(x), 1.0, 1.0}, vh, s));
-                WD_CUDA_TRY(cudaMemsetAsync(xs, 0, hx, s));
-            } else {
-                WD_TRY(run_blas(ctx, OpFlushX<PX, PS>{F64(x), FX(xs), FS(ps), d + 2}, vh, s));
-            }
             // an update that the iterated residual's convergence triggered is a
             // convergence check: FP64 directly, as are all updates after a failed check
             const bool check = r2_new <= stop2;
             const int op = (check || fp64_only) ? WD_F64 : outer;
-            WD_TRY(true_residual(op, vh, x, b, r, ax, d + 4, mdagm_outer, blas));
+            if constexpr (PS == PREC_F64) {
+                WD_TRY(run_blas(ctx, OpAxpby<PX, PREC_F64, true>{FX(xs), F64(x), 1.0, 1.0}, vh, s));
+                WD_CUDA_TRY(cudaMemsetAsync(xs, 0, hx, s));
+            } else if (op == WD_DF) {
+                WD_TRY(run_blas(ctx, OpFlushX<PX, PS, true>{F64(x), FX(xs), FS(ps), field_ref<PREC_DF>(r, vh), d + 2}, vh, s));
+            } else {
+                WD_TRY(run_blas(ctx, OpFlushX<PX, PS, false>{F64(x), FX(xs), FS(ps), {}, d + 2}, vh, s));
+            }
+            WD_TRY(true_residual<PS>(op, vh, x, b, rs, r, PS != PREC_F64, ax, d + 4, mdagm_outer, blas));
             WD_TRY(read_scalars(ctx, 4, 1, s));
             r2_true = h[4];
             ++st.reliable_updates;
             if (r2_true <= stop2 && op != WD_F64) {
                 // the double-word residual meets the target: only the FP64 one may end the solve
-                WD_TRY(true_residual(WD_F64, vh, x, b, r, ax, d + 4, mdagm_outer, blas));
+                WD_TRY(true_residual<PS>(WD_F64, vh, x, b, rs, r, false, ax, d + 4, mdagm_outer, blas));
                 WD_TRY(read_scalars(ctx, 4, 1, s));
                 r2_true = h[4];
                 ++st.reliable_updates;
@@ -184,7 +185,6 @@ int cg_run(wd_ctx *ctx, const wd_gauge *g, double mass, char *x, const char *b, 
                 status = set_error(WD_ENOCONV, "true residual is not finite at iteration %d", it);
                 break;
             }
-            WD_TRY(run_blas(ctx, OpConvert<PS, PREC_F64>{FS(rs), F64(r)}, vh, s));
             if (PS != PREC_F64)   // |r|^2 of the next step length
                 WD_CUDA_TRY(cudaMemcpyAsync(d, d + 4, sizeof(double), cudaMemcpyDeviceToDevice, s));
             r2_new = r2_true;
@@ -205,7 +205,7 @@ int cg_run(wd_ctx *ctx, const wd_gauge *g, double mass, char *x, const char *b, 
     }
     if (!converged && status == WD_OK) {
         WD_TRY(run_blas(ctx, OpAxpby<PX, PREC_F64, true>{FX(xs), F64(x), 1.0, 1.0}, vh, s));
-        WD_TRY(true_residual(WD_F64, vh, x, b, r, ax, d + 4, mdagm_outer, blas));
+        WD_TRY(true_residual<PS>(WD_F64, vh, x, b, rs, r, false, ax, d + 4, mdagm_outer, blas));
         WD_TRY(read_scalars(ctx, 4, 1, s));
         r2_true = h[4];
         status = set_error(WD_ENOCONV, "CG did not converge in %d iterations (relative residual %.3e)", it,

@@ -144,8 +144,8 @@ template <int PS> int iteration(const wd_ctx *ctx, GSolve &q)
                              CgFields{q.ps, q.rs, q.tso, q.tse, q.site, q.scal, q.red.partials, q.red.ticket}, q.s);
 }
 
-// r = b - A x (FP64; A applied in precision op, FP64 or double-word FP32);
-// r_lo = r; |r|^2 -> h[7] (asynchronous).
+// r_lo = b - A x (A applied in precision op, FP64 or double-word FP32: x in
+// double-word form is in q.r then); its FP64 |r|^2 -> h[7] (asynchronous).
 template <int PS> int residual_reseed(const wd_ctx *ctx, GSolve &q, int op)
 {
     const int vh = q.vh;
@@ -153,9 +153,8 @@ template <int PS> int residual_reseed(const wd_ctx *ctx, GSolve &q, int op)
         return mdagm(q.gauge, prec, q.opts.outer_recon, q.mass, in, out, q.t_o, q.t_e, q.s);
     };
     auto blas = [&](const auto &o) { return launch(ctx, o, vh, q.red, q.s); };
-    WD_TRY(true_residual(op, vh, (const char *)q.x, (const char *)q.b, q.r, q.ax, q.scal + 3, apply, blas));
-    WD_TRY(launch(ctx, OpConvert<PS, PREC_F64>{field_ref<PS>(q.rs, vh), field_ref<PREC_F64>(q.r, vh)}, vh, q.red,
-                  q.s));
+    WD_TRY(true_residual<PS>(op, vh, (const char *)q.x, (const char *)q.b, q.rs, q.r, true, q.ax, q.scal + 3, apply,
+                             blas));
     WD_CUDA_TRY(cudaMemcpyAsync(q.h + 7, q.scal + 3, sizeof(double), cudaMemcpyDeviceToHost, q.s));
     return WD_OK;
 }
@@ -165,10 +164,15 @@ template <int PS> int residual_reseed(const wd_ctx *ctx, GSolve &q, int op)
 template <int PS> int reliable_update(const wd_ctx *ctx, GSolve &q)
 {
     const int vh = q.vh;
-    WD_TRY(launch(ctx, OpFlushX<PREC_F32, PS>{field_ref<PREC_F64>(q.x, vh), field_ref<PREC_F32>(q.xs, vh),
-                                              field_ref<PS>(q.ps, vh), q.scal + 2}, vh, q.red, q.s));
+    const int op = q.update_fp64 ? WD_F64 : outer_prec_of(q.opts);
+    const FieldRef<PREC_F64> x = field_ref<PREC_F64>(q.x, vh);
+    const FieldRef<PREC_F32> xs = field_ref<PREC_F32>(q.xs, vh);
+    const FieldRef<PS> p = field_ref<PS>(q.ps, vh);
+    const FieldRef<PREC_DF> xd = field_ref<PREC_DF>(q.r, vh);
+    if (op == WD_DF) WD_TRY(launch(ctx, OpFlushX<PREC_F32, PS, true>{x, xs, p, xd, q.scal + 2}, vh, q.red, q.s));
+    else WD_TRY(launch(ctx, OpFlushX<PREC_F32, PS, false>{x, xs, p, xd, q.scal + 2}, vh, q.red, q.s));
     WD_CUDA_TRY(cudaMemsetAsync(q.scal + 2, 0, sizeof(double), q.s));
-    return residual_reseed<PS>(ctx, q, q.update_fp64 ? WD_F64 : outer_prec_of(q.opts));
+    return residual_reseed<PS>(ctx, q, op);
 }
 
 template <int PS> int init(const wd_ctx *ctx, GSolve &q, bool with_graph)
@@ -176,11 +180,12 @@ template <int PS> int init(const wd_ctx *ctx, GSolve &q, bool with_graph)
     const int vh = q.vh;
     auto F64 = [&](const void *p) { return field_ref<PREC_F64>(p, vh); };
     auto FS = [&](const void *p) { return field_ref<PS>(p, vh); };
-    WD_CUDA_TRY(cudaMemsetAsync(q.mem, 0, gs_footprint(vh, PS), q.s));
+    // what is read before it is written: x_lo, the scalars and the ticket (the
+    // end of the workspace; everything else is written first)
+    WD_CUDA_TRY(cudaMemsetAsync(q.xs, 0, (size_t)((char *)q.mem + gs_footprint(vh, PS) - q.xs), q.s));
     WD_TRY(launch(ctx, OpNorm2<PREC_F64>{F64(q.b), q.scal}, vh, q.red, q.s));
     WD_CUDA_TRY(cudaMemsetAsync(q.x, 0, (size_t)vh * 192, q.s));
-    WD_CUDA_TRY(cudaMemcpyAsync(q.r, q.b, (size_t)vh * 192, cudaMemcpyDeviceToDevice, q.s));
-    WD_TRY(launch(ctx, OpConvert<PS, PREC_F64>{FS(q.rs), F64(q.r)}, vh, q.red, q.s));
+    WD_TRY(launch(ctx, OpConvert<PS, PREC_F64>{FS(q.rs), F64(q.b)}, vh, q.red, q.s));
     WD_CUDA_TRY(cudaMemcpyAsync(q.ps, q.rs, half_field_bytes(vh, PS), cudaMemcpyDeviceToDevice, q.s));
     static const double inf = INFINITY;   // s[4] = inf: the first direction update gives p = r
     WD_CUDA_TRY(cudaMemcpyAsync(q.scal + 4, &inf, sizeof(double), cudaMemcpyHostToDevice, q.s));

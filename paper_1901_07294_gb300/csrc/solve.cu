@@ -98,8 +98,7 @@ int bicg_run(wd_ctx *ctx, const wd_gauge *g, double mass, char *x, const char *b
         WD_CUDA_TRY(cudaStreamSynchronize(s));
         return std::isfinite(b2) ? WD_OK : set_error(WD_EINVAL, "source is not finite");
     }
-    WD_CUDA_TRY(cudaMemcpyAsync(r, b, h64, cudaMemcpyDeviceToDevice, s));
-    WD_TRY(run_blas(ctx, OpConvert<PS, PREC_F64>{FS(rs), F64(r)}, vh, s));
+    WD_TRY(run_blas(ctx, OpConvert<PS, PREC_F64>{FS(rs), F64(b)}, vh, s));
     WD_CUDA_TRY(cudaMemsetAsync(xs, 0, hx, s));
     auto restart = [&]() -> int {
         WD_CUDA_TRY(cudaMemsetAsync(ps, 0, hs, s));
@@ -143,13 +142,13 @@ int bicg_run(wd_ctx *ctx, const wd_gauge *g, double mass, char *x, const char *b
         // convergence check: FP64 directly, as are all updates after a failed check
         const bool check = r2 <= stop2;
         const int op = (check || fp64_only) ? WD_F64 : outer;
-        WD_TRY(true_residual(op, vh, x, b, r, ax, d + 4, mhat_outer, blas));
+        WD_TRY(true_residual<PS>(op, vh, x, b, rs, r, false, ax, d + 4, mhat_outer, blas));
         WD_TRY(read_scal(ctx, 4, 1, s));
         r2_true = h[4];
         ++st.reliable_updates;
         if (r2_true <= stop2 && op != WD_F64) {
             // the double-word residual meets the target: only the FP64 one may end the solve
-            WD_TRY(true_residual(WD_F64, vh, x, b, r, ax, d + 4, mhat_outer, blas));
+            WD_TRY(true_residual<PS>(WD_F64, vh, x, b, rs, r, false, ax, d + 4, mhat_outer, blas));
             WD_TRY(read_scal(ctx, 4, 1, s));
             r2_true = h[4];
             ++st.reliable_updates;
@@ -165,7 +164,6 @@ int bicg_run(wd_ctx *ctx, const wd_gauge *g, double mass, char *x, const char *b
             status = set_error(WD_ENOCONV, "BiCGStab: true residual is not finite at iteration %d", it);
             break;
         }
-        WD_TRY(run_blas(ctx, OpConvert<PS, PREC_F64>{FS(rs), F64(r)}, vh, s));
         maxr = std::sqrt(r2_true);
         if (breakdown || !reliable) {
             r2_restart = r2_true;
@@ -176,7 +174,7 @@ int bicg_run(wd_ctx *ctx, const wd_gauge *g, double mass, char *x, const char *b
     }
     if (!converged && status == WD_OK) {
         WD_TRY(run_blas(ctx, OpAxpby<PX, PREC_F64, true>{FX(xs), F64(x), 1.0, 1.0}, vh, s));
-        WD_TRY(true_residual(WD_F64, vh, x, b, r, ax, d + 4, mhat_outer, blas));
+        WD_TRY(true_residual<PS>(WD_F64, vh, x, b, rs, r, false, ax, d + 4, mhat_outer, blas));
         WD_TRY(read_scal(ctx, 4, 1, s));
         r2_true = h[4];
         status = set_error(WD_ENOCONV, "BiCGStab did not converge in %d iterations (relative residual %.3e)", it,

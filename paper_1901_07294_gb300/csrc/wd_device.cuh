@@ -64,6 +64,23 @@ static __device__ __noinline__ float2 f64_split_rare(double v)
     return make_float2(h, __double2float_rn(v - (double)h));
 }
 
+static __device__ __noinline__ float f64_to_f32_rare(double v) { return (float)v; }
+
+// f64_to_f32: v rounded to FP32, to nearest even, in integer operations (an add
+// below bit 29 of the pattern, whose carry moves into the exponent) where the
+// result is a normal number and neither end of its range; the others, zero, inf
+// and NaN among them, out of line.
+__device__ __forceinline__ float f64_to_f32(double v)
+{
+    const unsigned long long b = (unsigned long long)__double_as_longlong(v);
+    const unsigned e = (unsigned)(b >> 52) & 0x7ffu;
+    if (e < 897u || e > 1148u) return f64_to_f32_rare(v);   // |v| < 2^-126 or >= 2^126
+    const unsigned long long r = b + 0x0fffffffull + ((b >> 29) & 1ull);
+    const unsigned er = (unsigned)(r >> 52) & 0x7ffu;
+    return __uint_as_float(((unsigned)(b >> 32) & 0x80000000u) | ((er - 896u) << 23) |
+                           ((unsigned)(r >> 29) & 0x7fffffu));
+}
+
 struct df {
     float hi, lo;
     df() = default;

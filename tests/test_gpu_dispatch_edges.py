@@ -127,3 +127,21 @@ def test_kept_workspaces_give_the_same_bits():
     q.wait(q.submit(dict(gauge=g, mass=0.2, tol=1e-10, x=x, b=b, inner_prec=wd.F16)))
     ctx.close()
     q.close()
+
+
+@pytest.mark.parametrize("dims", [(2, 2, 2, 2), (2, 4, 2, 6), (4, 6, 8, 10)])
+@pytest.mark.parametrize("inner", [wd.F64, wd.F32, wd.F16, wd.BF16])
+@pytest.mark.parametrize("outer", [wd.F64, wd.DF])
+@pytest.mark.parametrize("kw", [dict(), dict(use_graph=True), dict(reliable=False)], ids=["loop", "graph", "refine"])
+def test_reliable_updates_restart_from_the_true_residual(ctx, dims, inner, outer, kw):
+    """tol is 12 digits and delta 0.1, so that every inner precision restarts several times.  The
+    solver stops at 0.9 tol by its own FP64 residual, whose rounding (2^-53 times |A| |x| / |b| times
+    about 100 steps) is below 1e-13: the oracle's residual is then <= tol."""
+    U, b = synth.gauge(dims, seed=21), synth.even_spinor(dims, seed=22)
+    g = wd.Gauge(ctx, dims, U)
+    fb = pack_field(ctx, dims, wd.SITES_EVEN, wd.F64, b)
+    fx = wd.alloc_field(dims, wd.SITES_EVEN, wd.F64)
+    st = wd.cg_solve(ctx, g, 0.2, fx, fb, tol=1e-12, inner_prec=inner, outer_prec=outer, delta=0.1, **kw)
+    x = unpack_field(ctx, dims, wd.SITES_EVEN, wd.F64, fx)
+    rel = float(np.linalg.norm(b - oracle.mdagm(dims, U, 0.2, x)) / np.linalg.norm(b))
+    assert st["status"] == 0 and rel <= 1e-12, (st, rel)
