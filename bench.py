@@ -1109,17 +1109,21 @@ def _bicgstab_iteration_bytes(inner_prec, recon):
 
 def _cg_iteration_bytes(inner_prec, recon):
     """Bytes per even site that one CG iteration on Mhat^dagger Mhat moves by design
-    (every kernel's inputs read once, outputs written once): four even-odd hops
+    (every kernel's inputs read once, outputs written once).  FP64: four even-odd hops
     (spinor in and out, 8 links; the two Mhat hops also read their axpy term),
     Re<p, Ap> with alpha (p, Ap), the fused update (r and x read and written, Ap and
-    p read; |r|^2) and p = r + beta p.  That is 19 passes over inner-precision
-    fields, two over the x accumulator (FP32 for the reduced precisions, FP64 for
-    FP64) and four link sets.  Reliable updates and the final true residual come
-    on top."""
+    p read; |r|^2) and p = r + beta p: 19 passes over fields, two over the x
+    accumulator and four link sets.  The reduced precisions take the step length and
+    update r in the hops: four hops with 2, 3, 2 and 4 passes (the last reads its
+    axpy term and reads and writes r, and stores no A p), the update of x (FP32) and p
+    with 3 and two over x, and two sums over one FP32 number per site, each written
+    and read: 14 passes.  Reliable updates and the final true residual come on top."""
     fb = {0: 192, 1: 96, 2: 52, 3: 52}[inner_prec]
     link_b = {0: 8, 1: 4, 2: 2, 3: 2}[inner_prec] * recon * 8
     fx = 192 if inner_prec == 0 else 96
-    return 19 * fb + 4 * link_b + 2 * fx
+    if inner_prec == 0:
+        return 19 * fb + 4 * link_b + 2 * fx
+    return 14 * fb + 4 * link_b + 2 * fx + 16
 
 
 def _solve_section(wd, torch, ctx, peak):

@@ -8,8 +8,10 @@
 //                        the serving queue: one CUDA graph per group whose
 //                        device-side WHILE loop runs their iterations with
 //                        one shared-link launch per hop for all of them (4 hop
-//                        launches and 3 BLAS kernels, scalars in device
-//                        memory) until one needs its reliable update, which
+//                        launches, which also take the step lengths and
+//                        update r, one for x and p and one that sums |r|^2,
+//                        scalars in device memory) until one needs its
+//                        reliable update, which
 //                        the host enqueues on that solve's own stream while
 //                        the group goes on;
 //   WD_BATCH_PERSISTENT  one cooperative launch (all solves with the same

@@ -30,9 +30,10 @@ constexpr int GS_LAUNCH_CAP = 32;   // iterations at most per graph launch
 // Device scalar slots of a graph-driven solve: s[0] |r|^2, s[1] <p, A p>,
 // s[2] alpha of the last iteration, whose step is not yet in x (0: none
 // pending), s[3] true |r|^2, s[4] previous |r|^2,
-// s[5] beta = s[0] / s[4] for the next direction update, s[6] breakdown flag, s[8] max |r| since the last update, s[9] iterations in
-// this launch, s[10] iterations since the last update, s[11] iterations in
-// total, s[12] tol^2 |b|^2, s[13] delta, s[14] maxiter, s[15] GS_LAUNCH_CAP.
+// s[5] beta = s[0] / s[4] for the next direction update, s[6] breakdown flag,
+// s[8] max |r| since the last update, s[9] iterations in this launch, s[10]
+// iterations since the last update, s[11] iterations in total, s[12]
+// tol^2 |b|^2, s[13] delta, s[14] maxiter, s[15] GS_LAUNCH_CAP.
 constexpr int GS_NSCAL = 16;
 
 // One solve's bookkeeping after an iteration: max |r| since the last update,
