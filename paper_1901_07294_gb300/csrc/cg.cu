@@ -197,10 +197,13 @@ int cg_run(wd_ctx *ctx, const wd_gauge *g, double mass, char *x, const char *b, 
             }
         }
         const double beta = r2_new / r2;
-        if (PS == PREC_F64 || update)   // p = r + beta p; with x += alpha p unless an update has taken that step
-            WD_TRY(run_blas(ctx, OpAxpby<PS, PS>{FS(rs), FS(ps), 1.0, beta}, vh, s));
-        else
-            WD_TRY(run_blas(ctx, OpXp<PX, PS>{FX(xs), FS(rs), FS(ps), d + 2, nullptr, beta}, vh, s));
+        // p = r + beta p; with x += alpha p unless an update has taken that step
+        bool with_x = false;
+        if constexpr (PS != PREC_F64) {
+            with_x = !update;
+            if (with_x) WD_TRY(run_blas(ctx, OpXp<PS>{FX(xs), FS(rs), FS(ps), d + 2, nullptr, beta}, vh, s));
+        }
+        if (!with_x) WD_TRY(run_blas(ctx, OpAxpby<PS, PS>{FS(rs), FS(ps), 1.0, beta}, vh, s));
         r2 = r2_new;
     }
     if (!converged && status == WD_OK) {

@@ -180,8 +180,8 @@ template <int PS> __global__ void __launch_bounds__(BLAS_THREADS) gg_xp_kernel(c
     const size_t hs = half_bytes_p<PS>(vh), h32 = half_bytes_p<PREC_F32>(vh);
     for (int t = blockIdx.y; t < T->n; t += gridDim.y) {
         const GMember &m = T->m[T->idx[t]];
-        blas_body(OpXp<PREC_F32, PS>{FieldRef<PREC_F32>{m.xs, h32, vh}, FieldRef<PS>{m.f[GF_RS], hs, vh},
-                                     FieldRef<PS>{m.f[GF_PS], hs, vh}, m.scal + 2, m.scal + 5, 0.0}, vh, m.red);
+        blas_body(OpXp<PS>{FieldRef<PREC_F32>{m.xs, h32, vh}, FieldRef<PS>{m.f[GF_RS], hs, vh},
+                           FieldRef<PS>{m.f[GF_PS], hs, vh}, m.scal + 2, m.scal + 5, 0.0}, vh, m.red);
     }
 }
 

@@ -139,7 +139,7 @@ template <int PS> int iteration(const wd_ctx *ctx, GSolve &q)
 {
     const int vh = q.vh;
     auto FS = [&](const void *p) { return field_ref<PS>(p, vh); };
-    WD_TRY(launch(ctx, OpXp<PREC_F32, PS>{field_ref<PREC_F32>(q.xs, vh), FS(q.rs), FS(q.ps), q.scal + 2, q.scal + 5, 0.0},
+    WD_TRY(launch(ctx, OpXp<PS>{field_ref<PREC_F32>(q.xs, vh), FS(q.rs), FS(q.ps), q.scal + 2, q.scal + 5, 0.0},
                   vh, q.red, q.s));
     return cg_iteration_hops(q.gauge, PS, q.opts.inner_recon, q.mass,
                              CgFields{q.ps, q.rs, q.tso, q.tse, q.site, q.scal, q.red.partials, q.red.ticket}, q.s);
