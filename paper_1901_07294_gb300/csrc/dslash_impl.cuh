@@ -263,13 +263,13 @@ __device__ __forceinline__ void hop_dir(const char *in, const char *lblk, int vh
 // 16-bit storage: o = a x + acc at site i, with acc the sum already
 // weighted by the hop coefficient (hop_dir's wt); x is read as stored and its
 // per-site scale folded into a.
-template <int P, bool HAS_X>
+template <int P, bool HAS_X, bool LAST = false>
 __device__ __forceinline__ void value_weighted(const char *x, int vh, int i, float a, const cpx<float> (&acc)[4][3],
                                                float (&o)[24])
 {
     if constexpr (HAS_X) {
         unsigned u[12];
-        const float ax = a * Spinor<P>::load_words(x, vh, i, u);
+        const float ax = a * Spinor<P>::template load_words<LAST>(x, vh, i, u);
 #pragma unroll
         for (int s = 0; s < 4; ++s)
 #pragma unroll
@@ -298,8 +298,8 @@ __device__ __forceinline__ void store_weighted(const char *x, char *out, int vh,
 }
 
 // o = a x + b acc at site i of parity p, field at byte offset roff (16-bit
-// storage: acc already carries b).
-template <int P, bool HAS_X>
+// storage: acc already carries b).  LAST: x is not read again soon.
+template <int P, bool HAS_X, bool LAST = false>
 __device__ __forceinline__ void hop_value(const HopArgs &A, int p, int i, size_t roff,
                                           const cpx<typename Prec<P>::real> (&acc)[4][3],
                                           typename Prec<P>::real (&o)[24])
@@ -307,9 +307,9 @@ __device__ __forceinline__ void hop_value(const HopArgs &A, int p, int i, size_t
     using T = typename Prec<P>::real;
     const T a = (T)A.a, b = (T)A.b;
     if constexpr (Prec<P>::scaled) {
-        value_weighted<P, HAS_X>(HAS_X ? (p ? A.x[1] : A.x[0]) + roff : nullptr, A.vh, i, (float)A.a, acc, o);
+        value_weighted<P, HAS_X, LAST>(HAS_X ? (p ? A.x[1] : A.x[0]) + roff : nullptr, A.vh, i, (float)A.a, acc, o);
     } else if constexpr (HAS_X) {
-        Spinor<P>::load((p ? A.x[1] : A.x[0]) + roff, A.vh, i, o);
+        Spinor<P>::template load<LAST>((p ? A.x[1] : A.x[0]) + roff, A.vh, i, o);
 #pragma unroll
         for (int s = 0; s < 4; ++s)
 #pragma unroll

@@ -221,6 +221,11 @@ __device__ __forceinline__ uint4 ldg16(const void *p)
 {
     return __ldg(reinterpret_cast<const uint4 *>(p));
 }
+// As ldg16; LAST: with the streaming hint, for data that is not read again soon.
+template <bool LAST> __device__ __forceinline__ uint4 ldg16_last(const void *p)
+{
+    return LAST ? __ldcs(reinterpret_cast<const uint4 *>(p)) : ldg16(p);
+}
 // As ldg16, without allocating the line in L1.
 __device__ __forceinline__ uint4 ldg16_na(const void *p)
 {
@@ -410,25 +415,27 @@ template <int P> struct Spinor {
 
     // 16-bit types: the twelve storage words (spin s, colour c in word 3s+c,
     // real part low) and the per-site scale.
+    template <bool LAST = false>
     __device__ static __forceinline__ float load_words(const char *f, int vh, int i, unsigned (&u)[12])
     {
         static_assert(Prec<P>::scaled, "16-bit storage only");
         const float s = __ldg(reinterpret_cast<const float *>(f + (size_t)nplane * vh * 16) + i);
 #pragma unroll
         for (int k = 0; k < nplane; ++k) {
-            const uint4 w = ldg16(f + ((size_t)k * vh + i) * 16);
+            const uint4 w = ldg16_last<LAST>(f + ((size_t)k * vh + i) * 16);
             u[4 * k] = w.x; u[4 * k + 1] = w.y; u[4 * k + 2] = w.z; u[4 * k + 3] = w.w;
         }
         return s;
     }
 
+    template <bool LAST = false>
     __device__ static __forceinline__ void load(const char *f, int vh, int i, real (&v)[24])
     {
         float s = 1.0f;
         if (Prec<P>::scaled) s = __ldg(reinterpret_cast<const float *>(f + (size_t)nplane * vh * 16) + i);
 #pragma unroll
         for (int k = 0; k < nplane; ++k) {
-            uint4 w = ldg16(f + ((size_t)k * vh + i) * 16);
+            uint4 w = ldg16_last<LAST>(f + ((size_t)k * vh + i) * 16);
             unpack16<P>(w, v + k * Prec<P>::per16, s);
         }
     }
