@@ -157,12 +157,13 @@ def _check(status: int) -> None:
 # and (in the library) no tuning key while nothing has been tuned.
 @functools.lru_cache(maxsize=256)
 def _dims_array(dims):
-    return _DIMS(*[int(d) for d in dims])
+    return _DIMS(*dims)
 
 
 def _dims(dims):
-    """The C array of the extents (shared between calls: read only)."""
-    return _dims_array(tuple(dims))
+    """The C array of the extents (shared between calls: read only), kept by their values:
+    the elements themselves may be unhashable, or change between calls."""
+    return _dims_array(tuple(map(int, dims)))
 
 
 _raw_stream = _get_device = None
