@@ -10,7 +10,7 @@
 // The operations on a site and their order are those of hop_site's schedule 0.
 // One site per thread against this kernel, even-odd hop: 24^3 x 48 with the axpy
 // term 546 -> 522 us (467 at the pipe's rate), without 515 -> 507, 12^3 x 24 with it
-// 61.8 -> 42.1, 16^4 without 58.5 -> 54.0, 8^4 31.6 -> 12.2 us; full operator on 32^4
+// 61.8 -> 40.4, 16^4 without 58.5 -> 54.0, 8^4 31.6 -> 12.2 us; full operator on 32^4
 // 1628 -> 1625 us.
 // (Taking the two directions of a mu in one chain, s = U h + U^dagger h' for the
 // upper spins and 2 U h - s for the lower ones, needs 840 instructions and 505 us on

@@ -28,6 +28,8 @@
 #include <type_traits>
 #include <utility>
 
+#include "launch_rules.h"
+
 namespace wd {
 
 // Whether wd_launch uses programmatic dependent launch (read once).
@@ -127,11 +129,7 @@ inline int device_l2_bytes() { return device_attr<cudaDevAttrL2CacheSize>(129 <<
 // 0 if the grid fills the device anyway.
 inline size_t spread_smem(long long blocks, int resident, size_t static_bytes)
 {
-    const long long sms = device_sm_count(), k = (blocks + sms - 1) / sms;
-    if (k >= resident || k < 1) return 0;
-    const size_t per = (size_t)228 * 1024 / (size_t)k - 1024;   // 1 KB of each block's share is the system's
-    const size_t most = 227 * 1024;
-    return (per < most ? per : most) - static_bytes;
+    return spread_bytes(blocks, device_sm_count(), resident, static_bytes);
 }
 
 // Lets `kernel` use up to 227 KB of dynamic shared memory (less its static
@@ -143,7 +141,7 @@ template <typename K> inline cudaError_t allow_smem(K *kernel, std::atomic<unsig
     if (e != cudaSuccess) return e;
     const unsigned long long bit = 1ull << (dev & 63);
     if (done.load(std::memory_order_acquire) & bit) return cudaSuccess;
-    e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(227 * 1024 - static_bytes));
+    e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(BLOCK_SMEM - static_bytes));
     if (e == cudaSuccess) done.fetch_or(bit, std::memory_order_release);
     return e;
 }
