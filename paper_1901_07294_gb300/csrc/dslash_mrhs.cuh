@@ -118,6 +118,11 @@ __device__ __forceinline__ void hop_dir_smem(const char *in, int vh, int nb,
 // warp, so PAIRS takes each pair in a row; otherwise backward directions
 // first.  FP32 (12 fields, even-odd, 32^4) 380 us backward first, 372 in pairs;
 // FP16 on 16^3 x 32 46.0 and 46.7 us.
+// The projector with + comes first in each pair, that is the forward direction under
+// dagger: with the backward one first the 80-register FP32 builds of the dagger spill 208-220
+// bytes a thread (else 0-32).  us, dagger, 12 FP32 fields on 32^4 in z-strips, backward
+// directions first / in pairs, backward one first / in pairs, + first: even-odd 379 / 476
+// / 369, with the axpy term 416 / 522 / 410, full 740 / 980 / 736.
 template <int P, int SF, bool PAIRS>
 __device__ __forceinline__ void hop_site_smem(const char *in, int vh, int i, const int *nb,
                                               const typename LinkTile<typename Prec<P>::real>::V *lk, bool tneg,
@@ -130,7 +135,7 @@ __device__ __forceinline__ void hop_site_smem(const char *in, int vh, int i, con
     for (int sp = 0; sp < 4; ++sp)
 #pragma unroll
         for (int c = 0; c < 3; ++c) acc[sp][c] = {T(0), T(0)};
-    if constexpr (PAIRS) {
+    if constexpr (PAIRS && SF < 0) {
         hop_dir_smem<P, 0, SB, false>(in, vh, nb[128], lk + 4 * D, false, acc, wt);
         hop_dir_smem<P, 0, SF, true>(in, vh, nb[0], lk, false, acc, wt);
         hop_dir_smem<P, 1, SB, false>(in, vh, nb[160], lk + 5 * D, false, acc, wt);
@@ -139,6 +144,15 @@ __device__ __forceinline__ void hop_site_smem(const char *in, int vh, int i, con
         hop_dir_smem<P, 2, SF, true>(in, vh, nb[64], lk + 2 * D, false, acc, wt);
         hop_dir_smem<P, 3, SB, false>(in, vh, nb[224], lk + 7 * D, ntb, acc, wt);
         hop_dir_smem<P, 3, SF, true>(in, vh, nb[96], lk + 3 * D, ntf, acc, wt);
+    } else if constexpr (PAIRS) {
+        hop_dir_smem<P, 0, SF, true>(in, vh, nb[0], lk, false, acc, wt);
+        hop_dir_smem<P, 0, SB, false>(in, vh, nb[128], lk + 4 * D, false, acc, wt);
+        hop_dir_smem<P, 1, SF, true>(in, vh, nb[32], lk + 1 * D, false, acc, wt);
+        hop_dir_smem<P, 1, SB, false>(in, vh, nb[160], lk + 5 * D, false, acc, wt);
+        hop_dir_smem<P, 2, SF, true>(in, vh, nb[64], lk + 2 * D, false, acc, wt);
+        hop_dir_smem<P, 2, SB, false>(in, vh, nb[192], lk + 6 * D, false, acc, wt);
+        hop_dir_smem<P, 3, SF, true>(in, vh, nb[96], lk + 3 * D, ntf, acc, wt);
+        hop_dir_smem<P, 3, SB, false>(in, vh, nb[224], lk + 7 * D, ntb, acc, wt);
     } else {
         hop_dir_smem<P, 0, SB, false>(in, vh, nb[128], lk + 4 * D, false, acc, wt);
         hop_dir_smem<P, 1, SB, false>(in, vh, nb[160], lk + 5 * D, false, acc, wt);
@@ -203,7 +217,7 @@ __device__ __forceinline__ void mrhs_store(const HopArgs &A, int p, int i, size_
 // block computes right-hand sides y, y + blockDim.y, ... from them, so links
 // cost 1/nrhs of their single-field traffic.  Spinors are read per field as in
 // hop_kernel.  blockDim = (32, RY).  MINB: resident blocks of 256 threads per SM
-// the kernel is compiled for: 3 (at most 80 registers, no spills) or, for small
+// the kernel is compiled for: 3 (at most 80 registers, at most 32 bytes spilt) or, for small
 // grids (mrhs_small), 2; FP64 needs twice the registers per complex number and is
 // left unbounded (1).
 //
