@@ -25,13 +25,7 @@ std::string hop_key(const wd_ctx *ctx, const HopArgs &A, int prec, int recon, in
     return buf;
 }
 
-// Default shape of the shared-link kernel: {threads, variant}.
-// Threads: 4 warps per block, or 3 where that takes at least a tenth fewer warp
-// passes over the fields (large grids, more than 4 fields; us, 128 / 96 threads:
-// 32^4 even-odd, FP32, 5 fields 186.6 / 177.9, 6 fields 207.0 / 197.2; 24^3 full, FP32, 9
-// 12-real 201 / 191, 10 fields 220 / 228; 24 x 18 x 26 x 18 full, 13 fields 177.3 / 187.5;
-// with fewer fields the links' staging counts and wants the warps: 20^4 full, 3
-// fields 42.4 / 44.5; small grids too: 12 x 14 x 10 x 18, 5 fields 11.6 / 12.9).
+// Default shape of the shared-link kernel: {threads (mrhs_threads), variant}.
 // Site order: a source spinor is read as t+ neighbour and again, 2 Lz slices
 // later, as t- neighbour.  Where what is touched in between exceeds about half of L2 the
 // slices are visited in the widest z-strips whose 2 w slices take no more than 0.4
@@ -42,9 +36,9 @@ std::string hop_key(const wd_ctx *ctx, const HopArgs &A, int prec, int recon, in
 static std::pair<int, int> mrhs_default(const HopArgs &A, int prec, int recon, int nrhs)
 {
     const long long blocks = (long long)((A.vh + 31) / 32) * A.nparity;
-    int threads = 128, variant = HOP_MRHS_VARIANT;
-    if (prec == WD_F64) return {threads, variant};   // bound by the FP64 pipe
-    if (nrhs > 4 && !mrhs_small(blocks, threads) && 10 * 3 * ((nrhs + 2) / 3) <= 9 * 4 * ((nrhs + 3) / 4)) threads = 96;
+    int variant = HOP_MRHS_VARIANT;
+    if (prec == WD_F64) return {128, variant};   // bound by the FP64 pipe
+    const int threads = mrhs_threads(blocks, nrhs, prec == WD_F32, device_sm_count());
     const double field = half_field_bytes(1, prec), link = link_block_bytes(1, link_prec(prec), recon);
     const double slice = (double)(A.L[0] / 2) * A.L[1] * A.nparity * (2 * nrhs * field + 8 / A.nparity * link);
     const double l2 = (double)device_l2_bytes();

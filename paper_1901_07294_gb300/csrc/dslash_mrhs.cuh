@@ -118,8 +118,8 @@ __device__ __forceinline__ void hop_dir_smem(const char *in, int vh, int nb,
 // warp, so PAIRS takes each pair in a row; otherwise backward directions
 // first.  FP32 (12 fields, even-odd, 32^4) 380 us backward first, 372 in pairs;
 // FP16 on 16^3 x 32 46.0 and 46.7 us.
-// The projector with + comes first in each pair, that is the forward direction under
-// dagger: with the backward one first the 80-register FP32 builds of the dagger spill 208-220
+// The projector with + comes first in an FP32 pair, that is the forward direction under
+// dagger: with the backward one first the 80-register builds of the dagger spill 208-220
 // bytes a thread (else 0-32).  us, dagger, 12 FP32 fields on 32^4 in z-strips, backward
 // directions first / in pairs, backward one first / in pairs, + first: even-odd 379 / 476
 // / 369, with the axpy term 416 / 522 / 410, full 740 / 980 / 736.
@@ -135,7 +135,7 @@ __device__ __forceinline__ void hop_site_smem(const char *in, int vh, int i, con
     for (int sp = 0; sp < 4; ++sp)
 #pragma unroll
         for (int c = 0; c < 3; ++c) acc[sp][c] = {T(0), T(0)};
-    if constexpr (PAIRS && SF < 0) {
+    if constexpr (PAIRS && (SF < 0 || Prec<P>::scaled)) {
         hop_dir_smem<P, 0, SB, false>(in, vh, nb[128], lk + 4 * D, false, acc, wt);
         hop_dir_smem<P, 0, SF, true>(in, vh, nb[0], lk, false, acc, wt);
         hop_dir_smem<P, 1, SB, false>(in, vh, nb[160], lk + 5 * D, false, acc, wt);
@@ -163,18 +163,6 @@ __device__ __forceinline__ void hop_site_smem(const char *in, int vh, int i, con
         hop_dir_smem<P, 2, SF, true>(in, vh, nb[64], lk + 2 * D, false, acc, wt);
         hop_dir_smem<P, 3, SF, true>(in, vh, nb[96], lk + 3 * D, ntf, acc, wt);
     }
-}
-
-// A grid of shared-link blocks (`threads` threads each) that is at most two waves
-// of the 128-register build: short launches gain more from a thread with its
-// loads in flight than from more warps (80 registers: half again as many).  us, 80
-// against 128 registers, direction pairs: 16^4 even-odd, 6 FP16 fields 15.0 / 12.8,
-// 8 FP32 fields 21.7 / 18.9; 8^2 x 16^2 full, 12 FP16 fields 17.5 / 12.5; 8^4
-// even-odd, 12 FP32 fields 7.9 / 6.5; beyond two waves the other way: 16^3 x 32
-// even-odd, 6 FP16 fields 22.6 / 24.2, full 46.7 / 52.3; 32^4, 12 FP32 fields 372 / 390.
-inline bool mrhs_small(long long blocks, int threads)
-{
-    return blocks * threads <= 2LL * 512 * device_sm_count();
 }
 
 // out = a x + b acc at site i of parity p for the field at byte offset roff
@@ -315,7 +303,7 @@ cudaError_t launch_hop_mrhs(const HopArgs &A, int nrhs, int threads, int zs, cud
     if (zs <= 0 || zs >= A.L[2]) zs = 0;
     const dim3 grid((unsigned)(per * A.nparity)), block(32, ry);
     if constexpr (P == PREC_F64) return wd_launch(hop_mrhs_kernel<P, RECON, DAG, HX, 1>, grid, block, 0, s, A, nrhs, zs);
-    else if (mrhs_small(grid.x, threads))
+    else if (mrhs_small(grid.x, threads, P == PREC_F32, device_sm_count()))
         return wd_launch(hop_mrhs_kernel<P, RECON, DAG, HX, 2>, grid, block, 0, s, A, nrhs, zs);
     else return wd_launch(hop_mrhs_kernel<P, RECON, DAG, HX, 3>, grid, block, 0, s, A, nrhs, zs);
 }

@@ -275,7 +275,7 @@ template <int PS> int build(const wd_ctx *ctx, GGroup &g)
     };
     using R12 = std::integral_constant<int, 12>;
     using R18 = std::integral_constant<int, 18>;
-    const bool small = mrhs_small(hgrid.x, GG_SUM_THREADS);
+    const bool small = mrhs_small(hgrid.x, GG_SUM_THREADS, g.prec == WD_F32, device_sm_count());
     if (g.recon == 12) small ? hops(R12{}, std::true_type{}) : hops(R12{}, std::false_type{});
     else small ? hops(R18{}, std::true_type{}) : hops(R18{}, std::false_type{});
     wd_launch(gg_control_kernel, dim3((unsigned)cg_parts(vh, BLAS_THREADS), (unsigned)GG_BLAS_ROWS), bblk, 0, g.s,

@@ -22,4 +22,41 @@ inline size_t spread_bytes(long long blocks, int sms, int resident, size_t stati
     return (per < BLOCK_SMEM ? per : BLOCK_SMEM) - static_bytes;
 }
 
+// ---- shared-link kernel: build and block size ---------------------------------
+// A grid of shared-link blocks (`threads` threads each, `sms` SMs) that is at most two
+// waves of the 128-register build: short launches gain more from a thread with its
+// loads in flight than from more warps (80 registers: half again as many).  us, 80
+// against 128 registers, 128 threads: 16^4 even-odd, 6 FP16 fields 15.0 / 12.8,
+// 8 FP32 fields 21.7 / 18.9; 8^2 x 16^2 full, 12 FP16 fields 17.5 / 12.5; 8^4
+// even-odd, 12 FP32 fields 7.9 / 6.5; beyond two waves the other way: 16^3 x 32
+// even-odd, 6 FP16 fields 22.6 / 24.2, full 46.7 / 52.3; 32^4, 12 FP32 fields 372 / 390.
+// 96 threads, 5 FP32 fields: 1440 blocks 24.0 / 20.9, 1536 (more than two waves) 24.8 / 24.8.
+// 16-bit storage: the builds take the directions in different orders, so the choice looks
+// at the lattice only; a field's bits do not depend on how many others are in the launch.
+inline bool mrhs_small(long long blocks, int threads, bool f32, int sms)
+{
+    return blocks <= 2LL * (512 / (f32 ? threads : 128)) * sms;
+}
+
+// Threads of an untuned launch for `nrhs` fields: 4 warps, or 3 where that takes at least
+// a tenth fewer warp passes over the fields (5, 6, 9, ... fields) and the grid is large
+// enough to profit (with 4 fields or less the links' staging counts and wants the warps:
+// 20^4 full, 3 fields 42.4 / 44.5).
+// FP32: where the three-warp grid is at most two waves of the 128-register build (even-odd,
+// 5 fields, us, 4 warps / 3: 1280 blocks 22.3 / 19.6, 1440 23.9 / 20.9), and beyond that where
+// it is fewer waves of the other build (6 fields: 1792 blocks, two waves each, 28.8 / 30.6;
+// 2016, three / two, 35.5 / 32.5; 2560, three each, 41.2 / 42.4; 32^4, 16,384, 207 / 197).
+// 16-bit: from 11 blocks per SM on (FP16, 6 fields: 1440 blocks 16.4 / 17.4, 1536 18.1 / 18.6, 1792
+// 21.4 / 20.6, 2304 27.9 / 26.9, 3888 44.8 / 42.5).
+inline int mrhs_threads(long long blocks, int nrhs, bool f32, int sms)
+{
+    if (nrhs <= 4 || 10 * 3 * ((nrhs + 2) / 3) > 9 * 4 * ((nrhs + 3) / 4) || mrhs_small(blocks, 128, f32, sms)) return 128;
+    if (!f32) return blocks >= 11LL * sms ? 96 : 128;
+    auto waves = [&](int threads) {
+        const long long fit = 768 / threads * (long long)sms;
+        return (blocks + fit - 1) / fit;
+    };
+    return mrhs_small(blocks, 96, f32, sms) || waves(96) < waves(128) ? 96 : 128;
+}
+
 } // namespace wd
