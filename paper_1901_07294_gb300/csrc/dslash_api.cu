@@ -59,8 +59,8 @@ static std::pair<int, int> mrhs_default(const HopArgs &A, int prec, int recon, i
 // FP32 ones with schedule 0 (24^3 x 48: 42.2 against 43.4 us for schedule 1), with the
 // axpy term and 18-real links on large lattices schedule 1 (24^3 x 48 47.3 / 45.1,
 // 32^4 70.0 / 67.4), and the 16-bit ones with the spin-paired kernel (schedule 0); FP64
-// (bound by the FP64 pipe) with three threads per site (128: the block size of an
-// open-boundary pass, which uses hop_kernel).
+// (bound by the FP64 pipe) with three threads per site or one (f64_three_threads; 128: the
+// block size of the latter and of an open-boundary pass, which uses hop_kernel).
 constexpr int HOP_LARGE = 300000;   // sites of one parity: 24^3 x 48 has 331,776, 16^3 x 32 65,536
 
 static std::pair<int, int> hop_default(const HopArgs &A, int prec, int recon, int nrhs)
@@ -68,7 +68,10 @@ static std::pair<int, int> hop_default(const HopArgs &A, int prec, int recon, in
     const bool large = A.vh >= HOP_LARGE, hx = A.x[0] != nullptr || A.x[1] != nullptr;
     if (prec == WD_DF) return {96, HOP_ROW_VARIANT};   // double-word: three threads per site
     if (nrhs > 1) return mrhs_default(A, prec, recon, nrhs);
-    if (prec == WD_F64) return {128, HOP_ROW_VARIANT};
+    if (prec == WD_F64) {
+        const long long blocks = (long long)((A.vh + 31) / 32) * A.nparity;
+        return {128, f64_three_threads(blocks, device_sm_count(), hx, recon) ? HOP_ROW_VARIANT : 0};
+    }
     if (prec == WD_F32) {
         if (A.nparity == 2) return {64, 1};
         return {64, large && hx && recon == 18 ? HOP_NA1_VARIANT : HOP_NA0_VARIANT};

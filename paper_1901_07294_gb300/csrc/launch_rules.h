@@ -22,6 +22,23 @@ inline size_t spread_bytes(long long blocks, int sms, int resident, size_t stati
     return (per < BLOCK_SMEM ? per : BLOCK_SMEM) - static_bytes;
 }
 
+// ---- FP64 hop: three threads per site, or one ----------------------------------
+// `blocks`: blocks of 32 sites (both parities of a full operator).  Three threads per site,
+// except where the kernel with one site per thread fills whole waves of two 128-thread
+// blocks per SM, that is 8 blocks of 32 sites on the busiest one, and has less to do at its
+// barriers' place: without the axpy term, and with 12-real links in the first such wave
+// (their rebuilt row leaves room for 5 blocks of 32 sites per SM, so 8 take two turns).
+// us, one thread per site / three, even-odd: 18 reals without the term, 1120 blocks 58.8 / 60.8,
+// 2400 121.8 / 120.5, 3600 176.4 / 179.2, 4752 234.4 / 237.3; with it, 1120 blocks 62.5 / 62.5; 12 reals
+// without, 1120 blocks 72.0 / 82.4, 2400 145.6 / 146.2, 4752 283.7 / 287.8; with it, 1120 76.3 / 84.1,
+// 2400 153.0 / 149.9.  Elsewhere: 12 reals with it, 64 blocks 40.3 / 15.1, 1024 76.0 / 66.5, 1280
+// 146.5 / 84.5, 10,368 659.8 / 629.9.
+inline bool f64_three_threads(long long blocks, int sms, bool has_x, int recon)
+{
+    const long long k = (blocks + sms - 1) / sms;
+    return !((k % 8 == 0 && !has_x) || (k == 8 && recon == 12));
+}
+
 // ---- shared-link kernel: build and block size ---------------------------------
 // A grid of shared-link blocks (`threads` threads each, `sms` SMs) that is at most two
 // waves of the 128-register build: short launches gain more from a thread with its

@@ -1,0 +1,52 @@
+"""The untuned launch shape against its alternatives, where the rule that picks it turns."""
+import pytest
+
+import paper_1901_07294_gb300 as wd
+import synth
+from tests._gpu import pack_field
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def ctx():
+    return wd.Context(0)
+
+
+def _us(call, shapes):
+    """Best of seven rounds of 20 calls for each shape, taken in turn."""
+    import torch
+    best = {s: float("inf") for s in shapes}
+    for _ in range(7):
+        for s in shapes:
+            call(s)
+            e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            e0.record()
+            for _ in range(20):
+                call(None)
+            e1.record()
+            e1.synchronize()
+            best[s] = min(best[s], e0.elapsed_time(e1) * 50)
+    return best
+
+
+# blocks of 32 sites per SM (152): 6.7, 7.4, 8.4 and 15.8
+@pytest.mark.parametrize("dims", [(16, 16, 16, 16), (16, 14, 20, 16), (16, 16, 16, 20), (20, 20, 16, 24)])
+@pytest.mark.parametrize("recon", [18, 12])
+@pytest.mark.parametrize("with_x", [False, True])
+def test_f64_default_is_within_a_few_percent_of_both_layouts(ctx, dims, recon, with_x):
+    """One thread per site against three differs by up to 1.7x here; 6 % leaves room for the clock."""
+    g = wd.Gauge(ctx, dims, synth.gauge(dims, seed=478))
+    fin, x = (pack_field(ctx, dims, s, wd.F64, synth.spinor(dims, seed=490)) for s in (wd.SITES_ODD, wd.SITES_EVEN))
+    out = wd.alloc_field(dims, wd.SITES_EVEN, wd.F64)
+
+    def call(shape):
+        if shape is not None:
+            wd.tune_clear(ctx)
+            if shape != "default":
+                wd.tune_set_dslash(ctx, g, wd.F64, recon, False, with_x, 1, *shape)
+        wd.dslash_eo_apply(ctx, g, out, fin, x if with_x else None, 0, 4.1, -0.06, prec=wd.F64, recon=recon)
+
+    t = _us(call, ["default", (128, 0), (96, 15)])
+    wd.tune_clear(ctx)
+    assert t["default"] <= 1.06 * min(t.values()), t
