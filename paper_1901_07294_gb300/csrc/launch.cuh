@@ -123,10 +123,10 @@ inline int device_l2_bytes() { return device_attr<cudaDevAttrL2CacheSize>(129 <<
 
 // Dynamic shared memory that keeps a grid of less than a full wave evenly
 // spread.  A kernel dispatched while its predecessor's last blocks run finds
-// some SMs free and fills them to their limit, so a grid of, say, 6.7 blocks per
+// some SMs free and fills them to their limit, so a grid of, say, 4.3 blocks per
 // SM of a kernel that fits 8 ends up with 8 on some SMs and the others idle; asking for so
-// much shared memory that only ceil(blocks / SMs) fit gives every SM its share.
-// 0 if the grid fills the device anyway.
+// much shared memory that only ceil(blocks / SMs) fit gives every SM its share
+// (spread_bytes says when).
 inline size_t spread_smem(long long blocks, int resident, size_t static_bytes)
 {
     return spread_bytes(blocks, device_sm_count(), resident, static_bytes);

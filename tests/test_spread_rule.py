@@ -32,9 +32,11 @@ def test_as_many_blocks_fit_as_the_grid_needs(tmp_path):
     assert len(rows) > 1000
     for static, sms, resident, blocks, dyn in rows:
         need = -(-blocks // sms)
-        if need >= resident:
+        if need >= resident or 2 * need <= resident:   # fills the device, or two grids fit side by side
             assert dyn == 0
             continue
         total = -(-(static + dyn + 1024) // 128) * 128
         assert static + dyn <= 227 * 1024
-        assert (228 * 1024) // total == need, (static, sms, resident, blocks, dyn)
+        # (seven blocks: six fit, measured the same alone and better beside other streams)
+        assert (228 * 1024) // total == (6 if need == 7 else need), (static, sms, resident, blocks, dyn)
+        assert (228 * 1024) // (total - 128) > (6 if need == 7 else need)   # no more than that takes
