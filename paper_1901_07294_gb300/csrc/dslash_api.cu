@@ -70,7 +70,7 @@ static std::pair<int, int> hop_default(const HopArgs &A, int prec, int recon, in
     if (nrhs > 1) return mrhs_default(A, prec, recon, nrhs);
     if (prec == WD_F64) {
         const long long blocks = (long long)((A.vh + 31) / 32) * A.nparity;
-        return {128, f64_three_threads(blocks, device_sm_count(), hx, recon) ? HOP_ROW_VARIANT : 0};
+        return {128, f64_three_threads(blocks, device_sm_count(), recon) ? HOP_ROW_VARIANT : 0};
     }
     if (prec == WD_F32) {
         if (A.nparity == 2) return {64, 1};

@@ -31,19 +31,19 @@ inline size_t spread_bytes(long long blocks, int sms, int resident, size_t stati
 
 // ---- FP64 hop: three threads per site, or one ----------------------------------
 // `blocks`: blocks of 32 sites (both parities of a full operator).  Three threads per site,
-// except where the kernel with one site per thread fills whole waves of two 128-thread
-// blocks per SM, that is 8 blocks of 32 sites on the busiest one, and has less to do at its
-// barriers' place: without the axpy term, and with 12-real links in the first such wave
-// (their rebuilt row leaves room for 5 blocks of 32 sites per SM, so 8 take two turns).
-// us, one thread per site / three, even-odd: 18 reals without the term, 1120 blocks 58.8 / 60.8,
-// 2400 121.8 / 120.5, 3600 176.4 / 179.2, 4752 234.4 / 237.3; with it, 1120 blocks 62.5 / 62.5; 12 reals
-// without, 1120 blocks 72.0 / 82.4, 2400 145.6 / 146.2, 4752 283.7 / 287.8; with it, 1120 76.3 / 84.1,
-// 2400 153.0 / 149.9.  Elsewhere: 12 reals with it, 64 blocks 40.3 / 15.1, 1024 76.0 / 66.5, 1280
-// 146.5 / 84.5, 10,368 659.8 / 629.9.
-inline bool f64_three_threads(long long blocks, int sms, bool has_x, int recon)
+// except with 12-real links on grids that the kernel with one site per thread takes in one
+// even wave, two 128-thread blocks (8 of 32 sites) per SM: the rebuilt row leaves room for 5
+// three-thread blocks per SM, so 8 take two turns.  us, one thread per site / three, even-odd,
+// 12 reals without and with the axpy term: 64 blocks 38.6 / 15.1 and 40.3 / 15.1, 1024 71.9 /
+// 65.1 and 76.0 / 66.5, 1120 72.0 / 82.4 and 76.3 / 84.1, 1280 138.7 / 82.4 and 146.5 / 84.5, 2400
+// 145.6 / 146.2 and 153.0 / 149.9, 10,368 627 / 615 and 660 / 630.  18 reals: 64 blocks 31.8 /
+// 12.3 and 33.6 / 12.3, 1024 58.8 / 54.0 and 62.5 / 55.5, 1120 58.8 / 60.8 and 62.5 / 62.5, 1280
+// 114.0 / 68.7 and 122.4 / 70.6, 4752 234.4 / 237.3 and 248.4 / 244.1, 10,368 514 / 508 and 546 / 522;
+// one thread is 3 % faster on 1120 blocks without the term, but not beside other streams (graph
+// batch of eight 16^3 x 18 solves, 1152 blocks, FP64 updates: 23.6 ms, three threads 21.5).
+inline bool f64_three_threads(long long blocks, int sms, int recon)
 {
-    const long long k = (blocks + sms - 1) / sms;
-    return !((k % 8 == 0 && !has_x) || (k == 8 && recon == 12));
+    return recon == 18 || (blocks + sms - 1) / sms != 8;
 }
 
 // ---- shared-link kernel: build and block size ---------------------------------
