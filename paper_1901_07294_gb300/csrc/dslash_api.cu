@@ -52,20 +52,24 @@ static std::pair<int, int> mrhs_default(const HopArgs &A, int prec, int recon, i
     return {threads, variant};
 }
 
-// Untuned defaults, from tuning runs on GB300 (8^4 to 32^4): 64-thread blocks;
-// full operator: schedule 1, with 16-bit storage and 12-real links schedule 2 on
-// large lattices (us, schedule 1 / 2: 24^3 x 48 43.9 / 41.5, 32^4 66.1 / 62.2, 16^3 x 32 9.2 /
-// 9.5); even-odd hops (each link read once) load the links without L1 allocation,
-// FP32 ones with schedule 0 (24^3 x 48: 42.2 against 43.4 us for schedule 1), with the
-// axpy term and 18-real links on large lattices schedule 1 (24^3 x 48 47.3 / 45.1,
-// 32^4 70.0 / 67.4), and the 16-bit ones with the spin-paired kernel (schedule 0); FP64
-// (bound by the FP64 pipe) with three threads per site or one (f64_three_threads; 128: the
+// Untuned defaults, from tuning runs on GB300 (8^4 to 32^4): 64-thread blocks.
+// Full operator: schedule 1; with 16-bit storage and 12-real links schedule 2, which also
+// prefetches the backward links, once the call touches more than three quarters of L2 and
+// those links are no longer found there (FP16, us, schedule 1 / 2, without and with dagger:
+// 16^3 x 32 (26 MB) 9.2 / 9.2 and 8.9 / 9.4, 24^4 (66) 22.2 / 21.7 and 21.7 / 21.9, 24^3 x 32 (88)
+// 29.6 / 28.4 and 28.6 / 28.7, 32^2 x 16 x 32 (105) 34.5 / 33.0 and 33.6 / 33.4, 24^3 x 48 (133) 43.0 /
+// 40.8 and 41.7 / 41.2, 32^4 (210) 64.9 / 62.0 and 63.1 / 62.6; L2 129 MB).
+// Even-odd hops (each link read once) load the links without L1 allocation.  FP32: schedule
+// 0, but 1 with the axpy term and 18-real links (schedule 0 / 1: 12^3 x 24 4.39 / 4.28, 16^4 4.9
+// / 4.7, 16^3 x 32 7.7 / 7.3, 24^4 25.6 / 24.0, 24^3 x 32 30.8 / 31.3, 24^3 x 40 39.0 / 38.5, 24^3 x 48
+// 47.1 / 45.3, 32^4 70.0 / 67.9; without the term 16^3 x 32 7.2 / 7.4, 24^3 x 48 43.3 / 43.6; 12 reals
+// with it 16^3 x 32 6.4 / 6.5, 24^4 20.7 / 20.1, 24^3 x 48 37.3 / 37.4, 32^4 55.1 / 55.8).  16-bit: the
+// spin-paired kernel (schedule 0).
+// FP64 (bound by the FP64 pipe): three threads per site or one (f64_three_threads; 128: the
 // block size of the latter and of an open-boundary pass, which uses hop_kernel).
-constexpr int HOP_LARGE = 300000;   // sites of one parity: 24^3 x 48 has 331,776, 16^3 x 32 65,536
-
 static std::pair<int, int> hop_default(const HopArgs &A, int prec, int recon, int nrhs)
 {
-    const bool large = A.vh >= HOP_LARGE, hx = A.x[0] != nullptr || A.x[1] != nullptr;
+    const bool hx = A.x[0] != nullptr || A.x[1] != nullptr;
     if (prec == WD_DF) return {96, HOP_ROW_VARIANT};   // double-word: three threads per site
     if (nrhs > 1) return mrhs_default(A, prec, recon, nrhs);
     if (prec == WD_F64) {
@@ -74,10 +78,11 @@ static std::pair<int, int> hop_default(const HopArgs &A, int prec, int recon, in
     }
     if (prec == WD_F32) {
         if (A.nparity == 2) return {64, 1};
-        return {64, large && hx && recon == 18 ? HOP_NA1_VARIANT : HOP_NA0_VARIANT};
+        return {64, hx && recon == 18 ? HOP_NA1_VARIANT : HOP_NA0_VARIANT};
     }
     if (A.nparity == 1) return {64, HOP_SP0_VARIANT};
-    return {64, large && recon == 12 ? 2 : 1};
+    const double bytes = 2.0 * A.vh * (2 * half_field_bytes(1, prec) + 4 * link_block_bytes(1, link_prec(prec), recon));
+    return {64, recon == 12 && bytes > 0.75 * device_l2_bytes() ? 2 : 1};
 }
 
 int hop_launch_cfg(const HopArgs &A, int prec, int recon, int dagger, int nrhs, int threads, int variant,

@@ -14,13 +14,14 @@ def ctx():
 
 
 def _us(call, shapes):
-    """Best of seven rounds of 20 calls for each shape, taken in turn."""
+    """Best of seven rounds of 20 calls for each shape, taken in turn, behind a wait that hides their launches."""
     import torch
     best = {s: float("inf") for s in shapes}
     for _ in range(7):
         for s in shapes:
             call(s)
             e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            torch.cuda._sleep(300000)
             e0.record()
             for _ in range(20):
                 call(None)
@@ -50,3 +51,32 @@ def test_f64_default_is_within_a_few_percent_of_both_layouts(ctx, dims, recon, w
     t = _us(call, ["default", (128, 0), (96, 15)])
     wd.tune_clear(ctx)
     assert t["default"] <= 1.06 * min(t.values()), t
+
+
+# FP32 with the axpy term where schedule 1 is 6 % faster than schedule 0, and 16-bit 12-real operators
+# either side of three quarters of L2, where schedule 2 is 2 % slower and 5 % faster than schedule 1
+@pytest.mark.parametrize("dims,prec,recon,full,dagger,shapes", [
+    ((16, 16, 16, 32), wd.F32, 18, False, False, [(64, 11), (64, 12)]),
+    ((24, 24, 24, 24), wd.F32, 18, False, True, [(64, 11), (64, 12)]),
+    ((16, 16, 16, 32), wd.F16, 12, True, True, [(64, 1), (64, 2)]),
+    ((24, 24, 24, 40), wd.F16, 12, True, False, [(64, 1), (64, 2)])])
+def test_schedule_default_is_the_faster_one(ctx, dims, prec, recon, full, dagger, shapes):
+    """Runs of one shape differ by up to 1 % here."""
+    g = wd.Gauge(ctx, dims, synth.gauge(dims, seed=479))
+    sites = (wd.SITES_FULL, wd.SITES_FULL) if full else (wd.SITES_ODD, wd.SITES_EVEN)
+    fin, x = (pack_field(ctx, dims, s, prec, synth.spinor(dims, seed=491)) for s in sites)
+    out = wd.alloc_field(dims, sites[1], prec)
+
+    def call(shape):
+        if shape is not None:
+            wd.tune_clear(ctx)
+            if shape != "default":
+                wd.tune_set_dslash(ctx, g, prec, recon, full, True, 1, *shape)
+        if full:
+            (wd.dslash_apply_dagger if dagger else wd.dslash_apply)(ctx, g, out, fin, 0.1, prec=prec, recon=recon)
+        else:
+            wd.dslash_eo_apply(ctx, g, out, fin, x, 0, 4.1, -0.06, dagger=dagger, prec=prec, recon=recon)
+
+    t = _us(call, ["default", *shapes])
+    wd.tune_clear(ctx)
+    assert t["default"] <= 1.02 * min(t.values()), t
