@@ -245,7 +245,11 @@ int wd_device_status(wd_ctx *ctx, int *code);
  * are written to `table`.  Synchronous.  Results of tuned and untuned
  * launches can differ in the last bits (the summation order of the eight
  * directions depends on the variant).  wd_tune_set_dslash pins a
- * configuration; wd_tune_clear forgets all of them. */
+ * configuration; wd_tune_clear forgets all of them.  The hops of a mixed-precision
+ * CG iteration that carry its vector work (all but the first) take the entry's
+ * block size, schedule (0 or 1) and way of loading the links; they have no builds
+ * of their own for 2, 4, 8 and 9, which run there as schedule 1, and with FP16 and
+ * BF16 they always run spin-paired. */
 typedef struct {
     int threads;
     int variant;

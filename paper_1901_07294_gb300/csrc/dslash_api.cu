@@ -102,11 +102,17 @@ int hop_launch_cfg(const HopArgs &A, int prec, int recon, int dagger, int nrhs, 
     return WD_OK;
 }
 
-int hop_launch(wd_ctx *ctx, const HopArgs &A, int prec, int recon, int dagger, int nrhs, cudaStream_t s)
+// {threads, variant} of a hop: the context's entry for its shape, else `def`.
+std::pair<int, int> hop_config(wd_ctx *ctx, const HopArgs &A, int prec, int recon, int nrhs, std::pair<int, int> def)
 {
     // the key of a launch is a string: 1 us to build, on a call of 3 us
-    auto cfg = hop_default(A, prec, recon, nrhs);
-    if (ctx->any_tuned.load(std::memory_order_acquire)) cfg = tuned_config(ctx, hop_key(ctx, A, prec, recon, nrhs), cfg);
+    if (!ctx->any_tuned.load(std::memory_order_acquire)) return def;
+    return tuned_config(ctx, hop_key(ctx, A, prec, recon, nrhs), def);
+}
+
+int hop_launch(wd_ctx *ctx, const HopArgs &A, int prec, int recon, int dagger, int nrhs, cudaStream_t s)
+{
+    const auto cfg = hop_config(ctx, A, prec, recon, nrhs, hop_default(A, prec, recon, nrhs));
     return hop_launch_cfg(A, prec, recon, dagger, nrhs, cfg.first, cfg.second, s);
 }
 

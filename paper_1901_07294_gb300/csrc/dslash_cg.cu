@@ -1,28 +1,58 @@
 // Host side of the CG iteration's hops (dslash_cg.cuh).
 #include "cg_iter.h"
 #include "dslash_cg.cuh"
+#include "dslash_launch.cuh"
 
 namespace wd {
 
 int hop_setup(const wd_gauge *g, int prec, int recon, HopArgs &A);
+std::pair<int, int> hop_config(wd_ctx *ctx, const HopArgs &A, int prec, int recon, int nrhs, std::pair<int, int> def);
 
 namespace {
 
-constexpr int CG_HOP_THREADS = 64;   // the untuned hops' block size
-
-template <int P, int RECON> cudaError_t launch_step(int step, const HopArgs &A, const CgHop &C, cudaStream_t s)
+// The launch shape is the context's entry for an even-odd hop of the same problem (tuned or
+// pinned): its block size and, of its variant, the schedule (0 or 1) and how the links are
+// loaded.  These hops have no builds of their own for schedule 2, the 3-block build (4), the
+// shared-memory window (8) and two sites per thread (9), which run as schedule 1; 16-bit
+// storage always runs spin-paired, schedule 0 with links loaded without L1 allocation and
+// schedule 1 with it.
+// Without an entry: 64 threads, links without L1 allocation, schedule 0, and 1 for FP32 with
+// the axpy term (a solve, ms, schedule 0 / 1, FP32: 16^4 4.85 / 4.74, 24^3 x 48 28.5 / 28.1, 32^4 41.5
+// / 41.2; 12 reals 16^4 4.80 / 4.68, 16^3 x 32 6.69 / 6.54, 24^3 x 48 24.9 / 25.0, 32^4 36.2 / 36.4; FP16,
+// spin-paired, 16^4 4.32 / 4.23, 24^3 x 32 12.9 / 13.2, 24^3 x 48 19.2 / 19.9).
+template <int P, int RECON, int PF, bool LNA>
+cudaError_t launch_step(int step, const HopArgs &A, const CgHop &C, int threads, cudaStream_t s)
 {
-    const int blocks = (A.vh + CG_HOP_THREADS - 1) / CG_HOP_THREADS;
-    const dim3 block(CG_HOP_THREADS);
-    if (step == CG_NORM) return wd_launch(hop_cg_kernel<P, RECON, CG_NORM>, dim3(blocks), block, 0, s, A, C, 0);
-    if (step == CG_RESID) return wd_launch(hop_cg_kernel<P, RECON, CG_RESID>, dim3(blocks), block, 0, s, A, C, 0);
-    const int parts = cg_parts(A.vh, CG_HOP_THREADS);
-    return wd_launch(hop_cg_kernel<P, RECON, CG_ALPHA>, dim3(parts + blocks), block, 0, s, A, C, parts);
+    const int blocks = (A.vh + threads - 1) / threads;
+    const dim3 block(threads);
+    if (step == CG_NORM) return wd_launch(hop_cg_kernel<P, RECON, CG_NORM, PF, LNA>, dim3(blocks), block, 0, s, A, C, 0);
+    if (step == CG_RESID)
+        return wd_launch(hop_cg_kernel<P, RECON, CG_RESID, PF, LNA>, dim3(blocks), block, 0, s, A, C, 0);
+    const int parts = cg_parts(A.vh, threads);
+    return wd_launch(hop_cg_kernel<P, RECON, CG_ALPHA, PF, LNA>, dim3(parts + blocks), block, 0, s, A, C, parts);
 }
 
-template <int P> cudaError_t launch_step(int recon, int step, const HopArgs &A, const CgHop &C, cudaStream_t s)
+template <int P, int RECON>
+cudaError_t launch_step(int step, const HopArgs &A, const CgHop &C, std::pair<int, int> cfg, cudaStream_t s)
 {
-    return recon == 12 ? launch_step<P, 12>(step, A, C, s) : launch_step<P, 18>(step, A, C, s);
+    const int v = cfg.second;
+    const bool first = v == 0 || v == HOP_NA0_VARIANT || v == HOP_SP0_VARIANT || v == HOP_ROW_VARIANT;   // schedule 0
+    if constexpr (Prec<P>::scaled) {
+        return first ? launch_step<P, RECON, 0, true>(step, A, C, cfg.first, s)
+                     : launch_step<P, RECON, 1, false>(step, A, C, cfg.first, s);
+    } else {
+        const bool na = v == HOP_NA0_VARIANT || v == HOP_NA1_VARIANT;
+        if (first) return na ? launch_step<P, RECON, 0, true>(step, A, C, cfg.first, s)
+                             : launch_step<P, RECON, 0, false>(step, A, C, cfg.first, s);
+        return na ? launch_step<P, RECON, 1, true>(step, A, C, cfg.first, s)
+                  : launch_step<P, RECON, 1, false>(step, A, C, cfg.first, s);
+    }
+}
+
+template <int P>
+cudaError_t launch_step(int recon, int step, const HopArgs &A, const CgHop &C, std::pair<int, int> cfg, cudaStream_t s)
+{
+    return recon == 12 ? launch_step<P, 12>(step, A, C, cfg, s) : launch_step<P, 18>(step, A, C, cfg, s);
 }
 
 int cg_hop(const wd_gauge *g, int prec, int recon, int step, const char *in, const char *x, char *out, double a,
@@ -37,11 +67,13 @@ int cg_hop(const wd_gauge *g, int prec, int recon, int step, const char *in, con
     A.parity0 = step == CG_ALPHA ? WD_ODD : WD_EVEN;
     A.a = a;
     A.b = b;
+    const int def = prec != WD_F32 ? HOP_SP0_VARIANT : x ? HOP_NA1_VARIANT : HOP_NA0_VARIANT;
+    const std::pair<int, int> cfg = hop_config(g->ctx, A, prec, recon, 1, {64, def});
     cudaError_t e;
     switch (prec) {
-    case WD_F16: e = launch_step<PREC_F16>(recon, step, A, C, s); break;
-    case WD_BF16: e = launch_step<PREC_BF16>(recon, step, A, C, s); break;
-    default: e = launch_step<PREC_F32>(recon, step, A, C, s); break;
+    case WD_F16: e = launch_step<PREC_F16>(recon, step, A, C, cfg, s); break;
+    case WD_BF16: e = launch_step<PREC_BF16>(recon, step, A, C, cfg, s); break;
+    default: e = launch_step<PREC_F32>(recon, step, A, C, cfg, s); break;
     }
     if (e != cudaSuccess) return set_error(WD_ECUDA, "hop kernel launch failed: %s", cudaGetErrorString(e));
     return WD_OK;

@@ -147,10 +147,10 @@ template <int P> struct CgResidStore {
     }
 };
 
-// One hop of the iteration with its share of the vector work: the kernel of the
-// untuned even-odd hops (links without L1 allocation; FP32: schedule 1 with the
-// axpy term, else 0; 16-bit storage: spin-paired, schedule 0).
-template <int P, int RECON, int STEP>
+// One hop of the iteration with its share of the vector work, in memory schedule PF (0
+// or 1) with or without L1 allocation for the links (LNA), as hop_kernel; 16-bit storage:
+// the spin-paired kernel.
+template <int P, int RECON, int STEP, int PF, bool LNA>
 __global__ void __launch_bounds__(256, 2) hop_cg_kernel(const HopArgs A, const CgHop C, const int nparts)
 {
     grid_dependency_enter();
@@ -170,8 +170,8 @@ __global__ void __launch_bounds__(256, 2) hop_cg_kernel(const HopArgs A, const C
     if (i >= A.vh) return;
     constexpr bool DAG = STEP != CG_NORM, HX = STEP != CG_ALPHA;
     auto run = [&](const auto &epi) {
-        if constexpr (Prec<P>::scaled) sp_site<P, RECON, DAG, HX, 0, true>(A, A.parity0, i, 0, epi);
-        else hop_site<P, RECON, DAG, HX, HX ? 1 : 0, false, true>(A, A.parity0, i, 0, epi);
+        if constexpr (Prec<P>::scaled) sp_site<P, RECON, DAG, HX, PF, LNA>(A, A.parity0, i, 0, epi);
+        else hop_site<P, RECON, DAG, HX, PF, false, LNA>(A, A.parity0, i, 0, epi);
     };
     if constexpr (STEP == CG_NORM) run(CgNormStore<P>{C.site});
     else if constexpr (STEP == CG_ALPHA) run(HopStore<P, false>{});
