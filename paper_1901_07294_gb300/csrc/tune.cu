@@ -106,15 +106,17 @@ int wd_tune_dslash(wd_ctx *ctx, const wd_gauge *g, int prec, int recon, int full
     cudaEvent_t e0, e1;
     cudaEventCreate(&e0);
     cudaEventCreate(&e1);
-    const int cand_threads[] = {64, 128, 192, 256};
+    // 96: for the shared-link variants, whose untuned default it is for some field counts
+    const int cand_threads[] = {64, 96, 128, 192, 256};
     int n = 0, best_t = 256, best_v = 1;
     double best_ms = 1e30;
     int rc = WD_OK;
-    for (int ti = 0; ti < 4 && rc == WD_OK; ++ti)
+    for (int ti = 0; ti < 5 && rc == WD_OK; ++ti)
         for (int v = 0; v <= HOP_MAX_VARIANT && rc == WD_OK; ++v) {
             const int th = cand_threads[ti];
             const int zs = hop_mrhs_strip(v);
             if (zs >= 0 && nrhs == 1) continue;
+            if (th == 96 && zs < 0) continue;
             if (zs > 0 && zs >= A.L[2]) continue;   // same as natural order
             if (v == HOP_RETIRED_VARIANT) continue;
             if ((v == HOP_SP1_VARIANT || v == HOP_SP0_VARIANT) && prec != WD_F16 && prec != WD_BF16) continue;
