@@ -14,7 +14,6 @@ where stated) in lexicographic order ``site = x + Lx*(y + Ly*(z + Lz*t))``.
 from __future__ import annotations
 
 import ctypes
-import functools
 import threading
 
 from . import _build
@@ -155,15 +154,24 @@ def _check(status: int) -> None:
 # another take 9.2 -> 3.9 us with torch's raw stream handle (a Stream object takes
 # 2.9 us to make), no lock around the loaded library, the lattice's C array kept,
 # and (in the library) no tuning key while nothing has been tuned.
-@functools.lru_cache(maxsize=256)
-def _dims_array(dims):
-    return _DIMS(*dims)
+_dims_kept = {}   # extents (plain integers) -> their C array, shared between calls: read only
 
 
 def _dims(dims):
-    """The C array of the extents (shared between calls: read only), kept by their values:
-    the elements themselves may be unhashable, or change between calls."""
-    return _dims_array(tuple(map(int, dims)))
+    """The C array of the extents.  Kept by their values: elements of other types may be
+    unhashable, or change between calls."""
+    if type(dims) is not tuple:
+        dims = tuple(map(int, dims))
+    try:
+        return _dims_kept[dims]
+    except (KeyError, TypeError):
+        pass
+    dims = tuple(map(int, dims))
+    arr = _DIMS(*dims)
+    if len(_dims_kept) >= 256:
+        _dims_kept.clear()
+    _dims_kept[dims] = arr
+    return arr
 
 
 _raw_stream = _get_device = None

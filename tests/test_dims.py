@@ -9,10 +9,12 @@ WANT = wd.field_bytes((8, 8, 8, 8), wd.SITES_FULL, wd.F32)
 
 def test_extents_are_read_at_each_call():
     """An extent held in a tensor or array may be changed in place between two calls."""
-    for d in ([torch.tensor(8) for _ in range(4)], [np.array(8) for _ in range(4)]):
-        assert wd.field_bytes(d, wd.SITES_FULL, wd.F32) == WANT
-        d[3][...] = 16
-        assert wd.field_bytes(d, wd.SITES_FULL, wd.F32) == 2 * WANT
+    for make in (torch.tensor, np.array):
+        for form in (list, tuple):
+            d = form(make(8) for _ in range(4))
+            assert wd.field_bytes(d, wd.SITES_FULL, wd.F32) == WANT
+            d[3][...] = 16
+            assert wd.field_bytes(d, wd.SITES_FULL, wd.F32) == 2 * WANT
 
 
 def test_extents_of_any_integer_like_type():
