@@ -139,9 +139,10 @@ int hop_setup(const wd_gauge *g, int prec, int recon, HopArgs &A)
 }
 
 int eo_hop(const wd_gauge *g, int prec, int recon, void *out, const void *in, const void *x, int p, double a,
-           double b, int dagger, cudaStream_t s)
+           double b, int dagger, cudaStream_t s, bool beside)
 {
     HopArgs A{};
+    A.beside = beside;
     WD_TRY(hop_setup(g, prec, recon, A));
     A.in[0] = A.in[1] = (const char *)in;
     A.x[0] = A.x[1] = (const char *)x;

@@ -195,7 +195,7 @@ cudaError_t launch_hop_f64_row(const HopArgs &A, int nrhs, cudaStream_t s)
     const int per = (A.vh + 31) / 32;
     const dim3 grid((unsigned)(per * A.nparity), (unsigned)nrhs);
     constexpr size_t fixed = sizeof(F64HalfTile<RECON>[2]);
-    const size_t pad = spread_smem((long long)grid.x * grid.y, f64_row_blocks<RECON>, fixed);
+    const size_t pad = spread_smem((long long)grid.x * grid.y, f64_row_blocks<RECON>, fixed, A.beside != 0);
     if (pad > 0) {
         static std::atomic<unsigned long long> allowed{0};
         const cudaError_t e = allow_smem(hop_f64_row_kernel<RECON, DAG, HX>, allowed, fixed);

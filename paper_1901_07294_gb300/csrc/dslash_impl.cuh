@@ -32,6 +32,7 @@ struct HopArgs {
     int topen;            // 1: open t boundary (a sub-domain): no hop crosses it (selects the TOPEN kernel)
     unsigned div_m[3];    // n / d for d = L[0]/2, L[1], L[2] as (n * m) >> s (set by hop_setup)
     int div_s[3];
+    int beside;           // 1: kernels of other streams are expected to run beside this one (host side: spread_bytes)
     int *status;          // device status word for asynchronous errors (bounded waits); may be NULL
     double a, b;
 };

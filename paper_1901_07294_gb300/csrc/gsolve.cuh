@@ -79,6 +79,7 @@ struct GSolve {
     const void *b = nullptr;
     wd_cg_opts opts{};
     int vh = 0, prec = WD_F32;
+    bool beside = false;   // other solves run beside it (a queue's requests)
     // resources
     cudaStream_t s = nullptr;
     cudaGraphExec_t exec = nullptr;
@@ -113,13 +114,13 @@ inline size_t gs_footprint(int vh, int prec)
 namespace gs_detail {
 
 inline int mdagm(const wd_gauge *g, int prec, int recon, double mass, const char *in, char *out, char *t_o,
-                 char *t_e, cudaStream_t s)
+                 char *t_e, cudaStream_t s, bool beside)
 {
     const double a = mass + 4.0, c = 1.0 / (4.0 * (mass + 4.0));
-    WD_TRY(eo_hop(g, prec, recon, t_o, in, nullptr, WD_ODD, 0.0, 1.0, 0, s));
-    WD_TRY(eo_hop(g, prec, recon, t_e, t_o, in, WD_EVEN, a, -c, 0, s));
-    WD_TRY(eo_hop(g, prec, recon, t_o, t_e, nullptr, WD_ODD, 0.0, 1.0, 1, s));
-    WD_TRY(eo_hop(g, prec, recon, out, t_o, t_e, WD_EVEN, a, -c, 1, s));
+    WD_TRY(eo_hop(g, prec, recon, t_o, in, nullptr, WD_ODD, 0.0, 1.0, 0, s, beside));
+    WD_TRY(eo_hop(g, prec, recon, t_e, t_o, in, WD_EVEN, a, -c, 0, s, beside));
+    WD_TRY(eo_hop(g, prec, recon, t_o, t_e, nullptr, WD_ODD, 0.0, 1.0, 1, s, beside));
+    WD_TRY(eo_hop(g, prec, recon, out, t_o, t_e, WD_EVEN, a, -c, 1, s, beside));
     return WD_OK;
 }
 
@@ -151,7 +152,7 @@ template <int PS> int residual_reseed(const wd_ctx *ctx, GSolve &q, int op)
 {
     const int vh = q.vh;
     auto apply = [&](int prec, const char *in, char *out) {
-        return mdagm(q.gauge, prec, q.opts.outer_recon, q.mass, in, out, q.t_o, q.t_e, q.s);
+        return mdagm(q.gauge, prec, q.opts.outer_recon, q.mass, in, out, q.t_o, q.t_e, q.s, q.beside);
     };
     auto blas = [&](const auto &o) { return launch(ctx, o, vh, q.red, q.s); };
     WD_TRY(true_residual<PS>(op, vh, (const char *)q.x, (const char *)q.b, q.rs, q.r, true, q.ax, q.scal + 3, apply,

@@ -127,9 +127,9 @@ inline int device_l2_bytes() { return device_attr<cudaDevAttrL2CacheSize>(129 <<
 // SM of a kernel that fits 8 ends up with 8 on some SMs and the others idle; asking for so
 // much shared memory that only ceil(blocks / SMs) fit gives every SM its share
 // (spread_bytes says when).
-inline size_t spread_smem(long long blocks, int resident, size_t static_bytes)
+inline size_t spread_smem(long long blocks, int resident, size_t static_bytes, bool beside)
 {
-    return spread_bytes(blocks, device_sm_count(), resident, static_bytes);
+    return spread_bytes(blocks, device_sm_count(), resident, static_bytes, beside);
 }
 
 // Lets `kernel` use up to 227 KB of dynamic shared memory (less its static

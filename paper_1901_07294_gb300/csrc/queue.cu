@@ -535,6 +535,7 @@ int rq_submit(rq_queue *q, const wd_solve_desc *d, uint64_t *ticket)
     r->gs.x = d->x_e;
     r->gs.b = d->b_e;
     r->gs.opts = d->opts;
+    r->gs.beside = true;   // its updates run beside its group's launches and other updates
     {
         std::lock_guard<std::mutex> lk(q->mu);
         if (q->stop) {

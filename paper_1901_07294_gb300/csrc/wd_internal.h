@@ -163,8 +163,9 @@ template <typename T> inline cudaError_t dev_malloc(const wd_ctx *ctx, T **p, si
 // code here; wd_device_status reads and clears it.
 inline int *ctx_status_word(const wd_ctx *c) { return c ? reinterpret_cast<int *>(c->d_ticket + 32) : nullptr; }
 // Even-odd hop on half fields: out_p = a x_p + b H^(d)_{p,1-p} in (see dslash_eo_apply).
+// beside: kernels of other streams are expected to run beside it.
 int eo_hop(const wd_gauge *g, int prec, int recon, void *out, const void *in, const void *x, int p, double a,
-           double b, int dagger, cudaStream_t s);
+           double b, int dagger, cudaStream_t s, bool beside = false);
 // Full-lattice hop on a full field: out = a in + b H in (both parities).
 int full_hop(const wd_gauge *g, int prec, int recon, void *out, const void *in, double a, double b, cudaStream_t s);
 // Launch configuration of a tunable kernel: the tuned one if the context has

@@ -18,7 +18,9 @@ int main() {
         for (int sms : {1, 148, 152})
             for (int res = 1; res <= 32; ++res)
                 for (int blocks = 1; blocks <= res * sms; blocks += blocks < 40 ? 1 : 37)
-                    std::printf("%%d %%d %%d %%d %%zu\\n", st, sms, res, blocks, wd::spread_bytes(blocks, sms, res, st));
+                    for (int beside = 0; beside < 2; ++beside)
+                        std::printf("%%d %%d %%d %%d %%d %%zu\\n", beside, st, sms, res, blocks,
+                                    wd::spread_bytes(blocks, sms, res, st, beside));
 }
 """
 
@@ -30,9 +32,9 @@ def test_as_many_blocks_fit_as_the_grid_needs(tmp_path):
     out = subprocess.run([str(tmp_path / "m")], check=True, capture_output=True, text=True).stdout
     rows = [tuple(map(int, l.split())) for l in out.splitlines()]
     assert len(rows) > 1000
-    for static, sms, resident, blocks, dyn in rows:
+    for beside, static, sms, resident, blocks, dyn in rows:
         need = -(-blocks // sms)
-        if need >= resident or 2 * need <= resident:   # fills the device, or two grids fit side by side
+        if need >= resident or (beside and 2 * need <= resident):   # fills the device, or leaves it to others
             assert dyn == 0
             continue
         total = -(-(static + dyn + 1024) // 128) * 128
