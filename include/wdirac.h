@@ -97,6 +97,14 @@ const char *wd_last_error(void);
 int wd_ctx_create(int device, wd_ctx **out);
 int wd_ctx_destroy(wd_ctx *ctx);
 
+/* Graph-driven cg_solve calls (use_graph = 1) and graph-mode batches leave their
+ * workspaces with the context, for later solves that need exactly as many bytes: at
+ * most 2 GiB and 32 of them, oldest given up first.  They are freed when an allocation
+ * of this library fails, when a queue's budget has no room for them, with the context,
+ * or by this call: all that are idle at once, their bytes to *freed (may be NULL).
+ * Callers whose other allocators need that memory call it after their solves. */
+int wd_ctx_trim(wd_ctx *ctx, size_t *freed);
+
 /* Bytes of one device field of `sites` (wd_sites) in precision `prec`,
  * times nrhs.  Errors: WD_EINVAL for bad dims, prec or nrhs < 1. */
 int wd_field_bytes(const int dims[4], int sites, int prec, int nrhs, size_t *out);
@@ -403,7 +411,8 @@ int wd_stream_mul(wd_ctx *ctx, int kind, size_t n, const double *x, const double
  * iterated residual has dropped by `delta` since the last update;
  * reliable = 0: iterative refinement with restarted inner solves to relative
  * residual `delta`.  Synchronous; uses a workspace owned by the context
- * (allocated on first use, grown when a larger lattice needs more).
+ * (allocated on first use, grown when a larger lattice needs more; with
+ * use_graph = 1 one of its own, kept as wd_ctx_trim says).
  * Returns WD_ENOCONV (stats still filled) if maxiter inner iterations pass
  * without convergence or the iteration breaks down. */
 typedef struct {
@@ -500,7 +509,8 @@ int wilson_solve(wd_ctx *ctx, const wd_gauge *g, double mass, void *x, const voi
  *                        several launches.
  * stats[k] receives solve k's statistics; `seconds` is the wall time of the
  * whole call.  Returns the first failure (WD_ENOCONV, WD_ETIMEOUT, ...).
- * Synchronous; allocates its workspace for the duration of the call. */
+ * Synchronous.  Graph mode leaves its workspaces with the context (wd_ctx_trim);
+ * persistent mode allocates its own for the duration of the call. */
 typedef enum { WD_BATCH_SEQUENTIAL = 0, WD_BATCH_GRAPH = 1, WD_BATCH_PERSISTENT = 2 } wd_batch_mode;
 
 typedef struct {
@@ -522,7 +532,9 @@ int cg_solve_batch(wd_ctx *ctx, int n, const wd_solve_desc *descs, int mode, wd_
  * are the caller's device buffers and must stay valid until the request's
  * result has been taken.  The scheduler admits waiting requests while fewer
  * than max_slots run and their workspace fits hbm_budget_bytes (first come
- * first served, a request that fits may pass one that does not).  Each
+ * first served, a request that fits may pass one that does not).  Idle workspaces,
+ * the queue's and those kept by the context, count against the budget when a request
+ * is admitted and are freed to fit it.  Each
  * admitted request has its own workspace and stream and joins the request
  * group of its gauge, inner precision and inner link format (up to 32
  * members; another group opens when one is full).  A group runs the
@@ -545,7 +557,8 @@ int cg_solve_batch(wd_ctx *ctx, int n, const wd_solve_desc *descs, int mode, wd_
  *              running (the request keeps running).
  *   rq_cancel: a waiting request ends at once with WD_ECANCELLED; a running one
  *              when its current launch or reliable update has finished.
- *   rq_destroy: finishes every submitted request, then stops and frees.
+ *   rq_destroy: finishes every submitted request, then stops and frees (its
+ *              workspaces too).
  * Times in wd_solve_result are seconds since rq_create.  A request whose
  * source is not finite ends with WD_EINVAL without affecting the others. */
 typedef struct rq_queue rq_queue;

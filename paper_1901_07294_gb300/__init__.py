@@ -44,6 +44,7 @@ _SIGS = {
     "wd_last_error": (ctypes.c_char_p, []),
     "wd_ctx_create": (_ip, [_ip, ctypes.POINTER(_vp)]),
     "wd_ctx_destroy": (_ip, [_vp]),
+    "wd_ctx_trim": (_ip, [_vp, ctypes.POINTER(_sz)]),
     "wd_field_bytes": (_ip, [_DIMS, _ip, _ip, _ip, ctypes.POINTER(_sz)]),
     "wd_pack": (_ip, [_vp, _DIMS, _ip, _ip, _vp, _vp, _vp]),
     "wd_pack_f32": (_ip, [_vp, _DIMS, _ip, _ip, _vp, _vp, _vp]),
@@ -218,6 +219,12 @@ class Context:
     @property
     def handle(self):
         return self._h
+
+    def trim(self) -> int:
+        """Free the workspaces that finished graph-driven solves left for later ones; their bytes."""
+        n = _sz()
+        _check(load().wd_ctx_trim(self._h, ctypes.byref(n)))
+        return int(n.value)
 
     def close(self):
         if self._h:

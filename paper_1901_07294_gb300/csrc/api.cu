@@ -397,16 +397,24 @@ void SolvePool::put(const Entry &e)
     }
 }
 
-void SolvePool::trim()
+size_t SolvePool::trim()
 {
+    size_t freed = 0;
     for (;;) {
         Entry old;
         {
             std::lock_guard<std::mutex> lk(mu);
-            if (!pop_oldest(old)) return;
+            if (!pop_oldest(old)) return freed;
         }
+        freed += old.bytes;
         free_entry(old);
     }
+}
+
+size_t SolvePool::held_bytes()
+{
+    std::lock_guard<std::mutex> lk(mu);
+    return held;
 }
 
 void SolvePool::close()
@@ -521,6 +529,16 @@ int wd_ctx_create(int device, wd_ctx **out)
     }
     load_tune_file(c);
     *out = c;
+    return WD_OK;
+}
+
+int wd_ctx_trim(wd_ctx *ctx, size_t *freed)
+{
+    clear_error();
+    if (!ctx) return set_error(WD_EINVAL, "ctx is NULL");
+    DeviceGuard dg(ctx->device);
+    const size_t n = ctx->solve_pool->trim();
+    if (freed) *freed = n;
     return WD_OK;
 }
 

@@ -541,7 +541,7 @@ int run_graph(wd_ctx *ctx, int n, const wd_solve_desc *d, wd_cg_stats *stats)
     size_t budget = 0;
     for (int k = 0; k < n; ++k) budget += gs_footprint(d[k].gauge->geo.Vh, d[k].opts.inner_prec);
     rq_queue *q = nullptr;
-    WD_TRY(rq_create(ctx, budget > 0 ? budget : 1, n > 0 ? n : 1, &q));
+    WD_TRY(rq_create_keep(ctx, budget > 0 ? budget : 1, n > 0 ? n : 1, true, &q));
     std::vector<uint64_t> tickets(n, 0);
     int rc = WD_OK, submitted = 0;
     for (int k = 0; k < n && rc == WD_OK; ++k, ++submitted) rc = rq_submit(q, &d[k], &tickets[k]);

@@ -69,7 +69,8 @@ struct QGroup {
 
 struct rq_queue {
     wd_ctx *ctx = nullptr;
-    std::shared_ptr<wd::SolvePool> solve_pool;   // the context's; gets the queue's idle workspaces at its end
+    std::shared_ptr<wd::SolvePool> solve_pool;   // the context's
+    bool keep = false;   // idle workspaces go to it at the queue's end (the queue of a batch)
     size_t budget = 0;
     int max_slots = 1;
     std::mutex mu;
@@ -90,7 +91,7 @@ struct rq_queue {
     // idle workspaces of finished requests, reused by requests of the same
     // footprint (scheduler thread only); they count against the budget
     std::vector<wd::SolvePool::Entry> pool;
-    size_t pool_bytes = 0;
+    size_t pool_bytes = 0, live = 0;   // bytes of idle workspaces and of those in use
     std::vector<QGroup *> groups;
     uint64_t group_launches = 0, group_members = 0;
 };
@@ -118,8 +119,8 @@ void finish(rq_queue *q, Req *r, int status)
 }
 
 // Workspace for an admitted request: an idle one of the same footprint if
-// there is one, else a new allocation after idle ones are freed until the
-// budget holds in-use plus idle memory.
+// there is one (the queue's, then the context's), else a new allocation after idle ones
+// are freed until the budget holds in-use plus idle memory, the context's included.
 int acquire(rq_queue *q, Req *r)
 {
     for (size_t k = 0; k < q->pool.size(); ++k)
@@ -127,6 +128,7 @@ int acquire(rq_queue *q, Req *r)
             r->gs.mem = q->pool[k].mem;
             r->gs.h = q->pool[k].h;
             r->gs.s = q->pool[k].s;
+            q->live += r->foot;
             q->pool_bytes -= r->foot;
             q->pool.erase(q->pool.begin() + (long)k);
             return WD_OK;
@@ -141,7 +143,18 @@ int acquire(rq_queue *q, Req *r)
         SolvePool::free_entry(q->pool.front());
         q->pool.erase(q->pool.begin());
     }
-    return gs_alloc(q->ctx, r->gs);
+    SolvePool::Entry e;
+    const bool kept = q->solve_pool->take(r->foot, e);
+    if (!q->keep && q->live + r->foot + q->pool_bytes + q->solve_pool->held_bytes() > q->budget) q->solve_pool->trim();
+    if (kept) {
+        r->gs.mem = e.mem;
+        r->gs.h = e.h;
+        r->gs.s = e.s;
+    } else {
+        WD_TRY(gs_alloc(q->ctx, r->gs));
+    }
+    q->live += r->foot;
+    return WD_OK;
 }
 
 // Returns a finished request's workspace to the pool.
@@ -172,6 +185,7 @@ void retire(rq_queue *q, Req *r, int rc)
         cudaEventDestroy(r->ev);
         r->ev = nullptr;
     }
+    q->live -= r->foot;
     if (rc == WD_ECUDA) gs_release(r->gs);
     else park(q, r);
     finish(q, r, rc != WD_OK ? rc : r->gs.status);
@@ -367,9 +381,11 @@ void scheduler(rq_queue *q)
             q->admitted++;
             const bool inject = q->fault_alloc_at > 0 && (int)q->admitted == q->fault_alloc_at;
             int rc = inject ? set_error(WD_ENOMEM, "injected allocation failure (WD_FAULT=alloc)") : acquire(q, r);
+            const bool acquired = rc == WD_OK;
             if (rc == WD_OK) rc = gs_bind(q->ctx, r->gs, false);
             if (rc == WD_OK) rc = join_group(q, r);
             if (rc != WD_OK) {
+                if (acquired) q->live -= r->foot;
                 gs_release(r->gs);
                 finish(q, r, rc);
                 continue;
@@ -460,7 +476,10 @@ void scheduler(rq_queue *q)
         delete G;
     }
     q->groups.clear();
-    for (auto &e : q->pool) q->solve_pool->put(e);
+    for (auto &e : q->pool) {
+        if (q->keep) q->solve_pool->put(e);
+        else SolvePool::free_entry(e);
+    }
     q->pool.clear();
     q->pool_bytes = 0;
 }
@@ -486,9 +505,7 @@ int check_request(const wd_solve_desc *d)
 
 using namespace wd;
 
-extern "C" {
-
-int rq_create(wd_ctx *ctx, size_t hbm_budget_bytes, int max_slots, rq_queue **out)
+int wd::rq_create_keep(wd_ctx *ctx, size_t hbm_budget_bytes, int max_slots, bool keep, rq_queue **out)
 {
     clear_error();
     if (!ctx || !out || max_slots < 1 || hbm_budget_bytes == 0) return set_error(WD_EINVAL, "bad arguments");
@@ -496,6 +513,7 @@ int rq_create(wd_ctx *ctx, size_t hbm_budget_bytes, int max_slots, rq_queue **ou
     if (!q) return set_error(WD_ENOMEM, "host allocation failed");
     q->ctx = ctx;
     q->solve_pool = ctx->solve_pool;
+    q->keep = keep;
     q->budget = hbm_budget_bytes;
     q->max_slots = max_slots;
     q->t0 = clk::now();
@@ -509,6 +527,13 @@ int rq_create(wd_ctx *ctx, size_t hbm_budget_bytes, int max_slots, rq_queue **ou
     }
     *out = q;
     return WD_OK;
+}
+
+extern "C" {
+
+int rq_create(wd_ctx *ctx, size_t hbm_budget_bytes, int max_slots, rq_queue **out)
+{
+    return rq_create_keep(ctx, hbm_budget_bytes, max_slots, false, out);
 }
 
 int rq_submit(rq_queue *q, const wd_solve_desc *d, uint64_t *ticket)

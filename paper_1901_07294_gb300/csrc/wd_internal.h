@@ -80,8 +80,10 @@ struct DeviceGuard {
 // Workspaces of finished graph-driven solves (device memory, pinned scalars and a
 // stream each), kept for later solves that need exactly as many bytes.
 // Allocating and freeing them took 0.2-0.5 ms of every solve (16^4 FP16 4.50 -> 4.28
-// ms, 24^3 x 48 20.2 -> 19.6; six 16^4 solves as a batch 14.9 -> 13.8).  At most MAX_ENTRIES and MAX_BYTES are held; all are given back when the
-// context is destroyed, or when an allocation of the library fails (dev_malloc).
+// ms, 24^3 x 48 20.2 -> 19.6; six 16^4 solves as a batch 14.9 -> 13.8).  At most MAX_ENTRIES
+// and MAX_BYTES are held; all are given back by wd_ctx_trim, when the context is
+// destroyed, when an allocation of the library fails (dev_malloc) and when a queue's
+// budget has no room for them.
 // Only idle workspaces are in here (their stream's work finished), handed out under
 // the lock to one solve at a time.  Shared by the context and its queues, so that
 // a queue closed after its context still finds it (closed: nothing is kept).
@@ -99,7 +101,8 @@ public:
     SolvePool() { idle.reserve(MAX_ENTRIES); }
     bool take(size_t bytes, Entry &e);
     void put(const Entry &e);   // kept, or freed if there is no room
-    void trim();                // frees all that is idle
+    size_t trim();              // frees all that is idle; returns its bytes
+    size_t held_bytes();
     void close();               // trim, and keep nothing from now on
     static void free_entry(const Entry &e);
 
@@ -174,6 +177,8 @@ std::pair<int, int> tuned_config(wd_ctx *ctx, const std::string &key, std::pair<
 void load_tune_file(wd_ctx *ctx);
 // Runs the autotuner for one hop shape unless the context already has it.
 int hop_ensure_tuned(wd_ctx *ctx, const wd_gauge *g, int prec, int recon, int full, int with_x);
+// rq_create for a batch: the queue's idle workspaces stay with the context when it ends.
+int rq_create_keep(wd_ctx *ctx, size_t hbm_budget_bytes, int max_slots, bool keep, rq_queue **out);
 // Solver workspace of at least `bytes` bytes (device), owned by the context.
 int ctx_workspace(wd_ctx *ctx, size_t bytes, char **out);
 // A second context-owned device buffer for drivers that call a solver (which
