@@ -118,12 +118,14 @@ __device__ __forceinline__ void hop_dir_smem(const char *in, int vh, int nb,
 // warp, so PAIRS takes each pair in a row; otherwise backward directions
 // first.  FP32 (12 fields, even-odd, 32^4) 380 us backward first, 372 in pairs;
 // FP16 on 16^3 x 32 46.0 and 46.7 us.
-// The projector with + comes first in an FP32 pair, that is the forward direction under
-// dagger: with the backward one first the 80-register builds of the dagger spill 208-220
-// bytes a thread (else 0-32).  us, dagger, 12 FP32 fields on 32^4 in z-strips, backward
+// PLUS: the projector with + comes first in each pair, that is the forward direction under
+// dagger (without dagger it is the backward one either way).  With the backward one first
+// the 80-register FP32 builds of the dagger spill 208-220 bytes a thread (else 0-32).  us, dagger, 12 FP32 fields on 32^4 in z-strips, backward
 // directions first / in pairs, backward one first / in pairs, + first: even-odd 379 / 476
-// / 369, with the axpy term 416 / 522 / 410, full 740 / 980 / 736.
-template <int P, int SF, bool PAIRS>
+// / 369, with the axpy term 416 / 522 / 410, full 740 / 980 / 736.  The 128-register build does
+// not spill and is up to 7 % faster with the backward one first (full, 8^4, 5 fields 5.1 / 5.4,
+// 12 x 14 x 10 x 18 15.2 / 15.6; even-odd with the axpy term, 16^4 19.5 / 20.3).
+template <int P, int SF, bool PAIRS, bool PLUS = false>
 __device__ __forceinline__ void hop_site_smem(const char *in, int vh, int i, const int *nb,
                                               const typename LinkTile<typename Prec<P>::real>::V *lk, bool tneg,
                                               const float wt, cpx<typename Prec<P>::real> (&acc)[4][3])
@@ -135,7 +137,7 @@ __device__ __forceinline__ void hop_site_smem(const char *in, int vh, int i, con
     for (int sp = 0; sp < 4; ++sp)
 #pragma unroll
         for (int c = 0; c < 3; ++c) acc[sp][c] = {T(0), T(0)};
-    if constexpr (PAIRS && (SF < 0 || Prec<P>::scaled)) {
+    if constexpr (PAIRS && (SF < 0 || !PLUS)) {
         hop_dir_smem<P, 0, SB, false>(in, vh, nb[128], lk + 4 * D, false, acc, wt);
         hop_dir_smem<P, 0, SF, true>(in, vh, nb[0], lk, false, acc, wt);
         hop_dir_smem<P, 1, SB, false>(in, vh, nb[160], lk + 5 * D, false, acc, wt);
@@ -234,7 +236,7 @@ __device__ __forceinline__ int mrhs_site(const HopArgs &A, int j, int zs)
     return off + sxy * (z + A.L[2] * t);
 }
 
-template <int P, int RECON, bool DAG, bool HAS_X, int MINB>
+template <int P, int RECON, bool DAG, bool HAS_X, int MINB, bool PLUS = false>
 __global__ void __launch_bounds__(256, MINB) hop_mrhs_kernel(const HopArgs A, const int nrhs, const int zs)
 {
     grid_dependency_enter();
@@ -290,7 +292,7 @@ __global__ void __launch_bounds__(256, MINB) hop_mrhs_kernel(const HopArgs A, co
         const char *in = (p ? A.in[1] : A.in[0]) + roff;
         const float wt = Prec<P>::scaled ? (float)A.b : 1.0f;   // 16-bit: b weights the terms
         cpx<T> acc[4][3];
-        hop_site_smem<P, SF, MINB == 2 || !Prec<P>::scaled>(in, vh, i, nb, &lk[0][0][s], A.tneg, wt, acc);
+        hop_site_smem<P, SF, MINB == 2 || !Prec<P>::scaled, PLUS>(in, vh, i, nb, &lk[0][0][s], A.tneg, wt, acc);
         mrhs_store<P, HAS_X>(A, p, i, roff, acc);
     }
 }
@@ -303,9 +305,17 @@ cudaError_t launch_hop_mrhs(const HopArgs &A, int nrhs, int threads, int zs, cud
     if (zs <= 0 || zs >= A.L[2]) zs = 0;
     const dim3 grid((unsigned)(per * A.nparity)), block(32, ry);
     if constexpr (P == PREC_F64) return wd_launch(hop_mrhs_kernel<P, RECON, DAG, HX, 1>, grid, block, 0, s, A, nrhs, zs);
-    else if (mrhs_small(grid.x, threads, P == PREC_F32, device_sm_count()))
-        return wd_launch(hop_mrhs_kernel<P, RECON, DAG, HX, 2>, grid, block, 0, s, A, nrhs, zs);
-    else return wd_launch(hop_mrhs_kernel<P, RECON, DAG, HX, 3>, grid, block, 0, s, A, nrhs, zs);
+    else {
+        const int sms = device_sm_count();
+        constexpr bool PLUS = P == PREC_F32 && DAG;
+        if (mrhs_small(grid.x, threads, P == PREC_F32, sms)) {
+            // the order of the sums by the lattice, as the 80-register build's in the same place
+            if (PLUS && !mrhs_small(grid.x, 128, true, sms))
+                return wd_launch(hop_mrhs_kernel<P, RECON, DAG, HX, 2, PLUS>, grid, block, 0, s, A, nrhs, zs);
+            return wd_launch(hop_mrhs_kernel<P, RECON, DAG, HX, 2>, grid, block, 0, s, A, nrhs, zs);
+        }
+        return wd_launch(hop_mrhs_kernel<P, RECON, DAG, HX, 3, PLUS>, grid, block, 0, s, A, nrhs, zs);
+    }
 }
 
 } // namespace wd

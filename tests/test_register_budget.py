@@ -21,7 +21,7 @@ namespace wd {
 
 @pytest.mark.skipif(not os.path.exists(NVCC), reason="no nvcc")
 def test_shared_link_fp32_builds_do_not_spill(tmp_path):
-    inst = [f"template __global__ void hop_mrhs_kernel<PREC_F32, {r}, {d}, {x}, 3>(HopArgs, int, int);"
+    inst = [f"template __global__ void hop_mrhs_kernel<PREC_F32, {r}, {d}, {x}, 3, {d}>(HopArgs, int, int);"
             for r in (18, 12) for d in ("false", "true") for x in ("false", "true")]
     (tmp_path / "k.cu").write_text(SRC % "\n".join(inst))
     r = subprocess.run([NVCC, "-gencode", "arch=compute_103a,code=sm_103a", "-O3", "-std=c++17", "-lineinfo",
