@@ -14,10 +14,11 @@ constexpr size_t SM_SMEM = 228 * 1024, BLOCK_SMEM = 227 * 1024, SYSTEM_SMEM = 10
 // even-odd hop alone, launches one after another, without / with: 648 blocks 59.4 / 40.4, 896
 // 61.2 / 47.9, 1024 62.1 / 55.5; 12-real links, 432 blocks 47.8 / 29.9.
 // 0 where the grid needs `resident` or more, and where other streams' kernels run beside it
-// and two such grids fit side by side (2 k <= resident): a successor dispatched early then
-// spreads as evenly (432 blocks 25.0 / 25.0), and the others' kernels fit in (a graph batch of
-// eight solves with FP64 updates, padded / not: 8^3 x 16 7.9 / 7.0 ms, 8^2 x 16^2 9.7 / 8.9, 12^3 x
-// 16 12.3 / 11.6).  Alone it is padded all the same: behind a kernel that leaves the SMs
+// and two such grids fit side by side with room left (2 k < resident): a successor
+// dispatched early then spreads as evenly (432 blocks 25.0 / 25.0), and the others' kernels
+// fit in (a graph batch of eight solves with FP64 updates, padded / not: 8^3 x 16 7.9 / 7.0 ms,
+// 8^2 x 16^2 9.7 / 8.9, 12^3 x 16 12.3 / 11.6; k = 4 of 8 is mixed: 8 x 20 x 10 x 20, 5 solves 10.0 /
+// 10.1, 8 solves 13.0 / 12.6, 10 x 12^2 x 24, 5 solves 9.9 / 10.4).  Alone it is padded all the same: behind a kernel that leaves the SMs
 // unevenly the blocks would stack up (host-driven BF16 CG with FP64 updates on 8^2 x 16^2, 256
 // blocks, 5.53 ms without, 5.26 with).
 // No more than keeps block k + 1 out, which leaves the rest to other streams; k = 7 gets 6:
@@ -26,7 +27,7 @@ constexpr size_t SM_SMEM = 228 * 1024, BLOCK_SMEM = 227 * 1024, SYSTEM_SMEM = 10
 inline size_t spread_bytes(long long blocks, int sms, int resident, size_t static_bytes, bool beside)
 {
     const long long k = (blocks + sms - 1) / sms;
-    if (k >= resident || k < 1 || (beside && 2 * k <= resident)) return 0;
+    if (k >= resident || k < 1 || (beside && 2 * k < resident)) return 0;
     const size_t next = (size_t)(k == 7 ? 7 : k + 1);   // blocks that must not fit
     const size_t per = (SM_SMEM / next / SMEM_UNIT + 1) * SMEM_UNIT - SYSTEM_SMEM;
     return (per < BLOCK_SMEM ? per : BLOCK_SMEM) - static_bytes;
