@@ -169,6 +169,9 @@ int wd_gauge_destroy(wd_gauge *g);
  * on double-word links (errors of order 2^-48 times the magnitudes of the
  * terms, FP32 instructions only: on a part whose FP64 rate is 1/64 of its
  * FP32 rate it replaces FP64 where 48 bits suffice).  out must not alias in.
+ * With nrhs >= 2 and no tuned entry a field's result does not depend on the other
+ * fields nor on how many there are (a single field, nrhs = 1, may be summed in
+ * another order of the directions).
  * Flop count: 1320 per site for H (Eq. (1): 8 directions of spin projection,
  * SU(3) x half-spinor and reconstruction).
  */

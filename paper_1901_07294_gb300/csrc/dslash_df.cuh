@@ -27,8 +27,9 @@
 namespace wd {
 
 constexpr int DF_ROW_THREADS = 96;
-// resident blocks per SM the register budget is set for (18-real links: 96
-// registers, 21 KB of shared memory; 12-real: 80)
+// resident blocks per SM the register budget is set for.  18-real links: at most 97
+// registers, of which the build takes 80, with 22.5 KB of shared memory, so that 8 blocks
+// are resident; 12-real: 80, 9.2 KB, 124 bytes spilt.
 template <int RECON> constexpr int df_row_blocks = RECON == 12 ? 8 : 7;
 
 // (h0, h1) = upper two spin components of (1 + S gamma_MU) psi for one colour,

@@ -464,7 +464,9 @@ void scheduler(rq_queue *q)
             }
             q->running.swap(keep);
         }
-        // nothing finished: wait briefly, or until a new request arrives
+        // nothing finished: wait briefly, or until a new request arrives.  Together with the
+        // timer slack this costs a third of one core while solves run (six 16^4 solves 4.8 ms
+        // of host time in 13.0, with 20 us and the default slack 3.5 in 16.2).
         if (!progress) {
             std::unique_lock<std::mutex> lk(q->mu);
             q->cv_work.wait_for(lk, std::chrono::microseconds(5),

@@ -26,13 +26,14 @@ def test_a_field_gets_the_same_bits_beside_any_number_of_others(ctx, dims, prec,
     g = wd.Gauge(ctx, dims, synth.gauge(dims, seed=177))
     nb = wd.field_bytes(dims, wd.SITES_ODD, prec)
     fin = torch.cat([pack_field(ctx, dims, wd.SITES_ODD, prec, synth.spinor(dims, seed=180 + k)) for k in range(6)])
-    res = {}
-    for n in (2, 4, 5, 6):
-        res[n] = wd.alloc_field(dims, wd.SITES_EVEN, prec, n)
-        wd.dslash_eo_apply(ctx, g, res[n], fin[:n * nb], None, 0, 0.0, 1.0, dagger=dagger, nrhs=n, prec=prec)
-    for n in (2, 4, 5):
-        assert torch.equal(res[n], res[6][:n * nb]), n
-    one = wd.alloc_field(dims, wd.SITES_EVEN, prec)
-    wd.dslash_eo_apply(ctx, g, one, fin[:nb], None, 0, 0.0, 1.0, dagger=dagger, prec=prec)
-    assert rel_max_err(unpack_field(ctx, dims, wd.SITES_EVEN, prec, res[6][:nb]),
-                       unpack_field(ctx, dims, wd.SITES_EVEN, prec, one)) < tol
+    x = torch.cat([pack_field(ctx, dims, wd.SITES_EVEN, prec, synth.spinor(dims, seed=180 + k)) for k in range(6)])
+    for a, b, xs in ((0.0, 1.0, None), (4.1, -0.06, x)):
+        def apply(out, n):
+            wd.dslash_eo_apply(ctx, g, out, fin[:n * nb], None if xs is None else xs[:n * nb], 0, a, b, dagger=dagger,
+                               nrhs=n, prec=prec)
+            return out
+        res = {n: apply(wd.alloc_field(dims, wd.SITES_EVEN, prec, n), n) for n in (1, 2, 4, 5, 6)}
+        for n in (2, 4, 5):
+            assert torch.equal(res[n], res[6][:n * nb]), n
+        assert rel_max_err(unpack_field(ctx, dims, wd.SITES_EVEN, prec, res[6][:nb]),
+                           unpack_field(ctx, dims, wd.SITES_EVEN, prec, res[1])) < tol
