@@ -60,11 +60,15 @@ static std::pair<int, int> mrhs_default(const HopArgs &A, int prec, int recon, i
 // 29.6 / 28.4 and 28.6 / 28.7, 32^2 x 16 x 32 (105) 34.5 / 33.0 and 33.6 / 33.4, 24^3 x 48 (133) 43.0 /
 // 40.8 and 41.7 / 41.2, 32^4 (210) 64.9 / 62.0 and 63.1 / 62.6; L2 129 MB).
 // Even-odd hops (each link read once) load the links without L1 allocation.  FP32: schedule
-// 0, but 1 with the axpy term and 18-real links (schedule 0 / 1: 12^3 x 24 4.39 / 4.28, 16^4 4.9
-// / 4.7, 16^3 x 32 7.7 / 7.3, 24^4 25.6 / 24.0, 24^3 x 32 30.8 / 31.3, 24^3 x 40 39.0 / 38.5, 24^3 x 48
-// 47.1 / 45.3, 32^4 70.0 / 67.9; without the term 16^3 x 32 7.2 / 7.4, 24^3 x 48 43.3 / 43.6; 12 reals
-// with it 16^3 x 32 6.4 / 6.5, 24^4 20.7 / 20.1, 24^3 x 48 37.3 / 37.4, 32^4 55.1 / 55.8).  16-bit: the
-// spin-paired kernel (schedule 0).
+// 0, but 1 with the axpy term and 18-real links, except on grids of 7 or 8 blocks per SM,
+// just under the one wave that is resident.  us, schedule 0 / 1, calls on several gauge
+// fields in turn: 12^3 x 24 6.1 / 5.2, 16^4 6.6 / 6.0, 14 x 16 x 20^2 8.0 / 7.7, 16^3 x 32 (7 blocks per
+// SM) 9.6 / 10.3, 20 x 26 x 6 x 44 (8) 10.2 / 10.7, 18^3 x 28 15.7 / 15.0, 20^3 x 24 17.3 / 16.5, 24^4 26.6
+// / 25.6, 24^3 x 32 31.1 / 31.4, 24^3 x 40 39.1 / 38.5, 24^3 x 48 47.1 / 45.5; on one field again and
+// again 16^4 4.9 / 4.7, 16^3 x 32 7.7 / 7.3, 20^3 x 24 14.3 / 12.9, 24^4 25.7 / 24.0, 24^3 x 48 47.2 / 45.7,
+// 32^4 70.0 / 67.9.  Without the term 16^3 x 32 7.2 / 7.4, 24^3 x 48 43.3 / 43.6; 12 reals with it
+// 16^3 x 32 6.4 / 6.5, 24^4 20.7 / 20.1, 24^3 x 48 37.3 / 37.4, 32^4 55.1 / 55.8.  16-bit: the spin-paired
+// kernel (schedule 0).
 // FP64 (bound by the FP64 pipe): three threads per site or one (f64_three_threads; 128: the
 // block size of the latter and of an open-boundary pass, which uses hop_kernel).
 static std::pair<int, int> hop_default(const HopArgs &A, int prec, int recon, int nrhs)
@@ -78,7 +82,8 @@ static std::pair<int, int> hop_default(const HopArgs &A, int prec, int recon, in
     }
     if (prec == WD_F32) {
         if (A.nparity == 2) return {64, 1};
-        return {64, hx && recon == 18 ? HOP_NA1_VARIANT : HOP_NA0_VARIANT};
+        const int sms = device_sm_count(), k = ((A.vh + 63) / 64 + sms - 1) / sms;
+        return {64, hx && recon == 18 && k != 7 && k != 8 ? HOP_NA1_VARIANT : HOP_NA0_VARIANT};
     }
     if (A.nparity == 1) return {64, HOP_SP0_VARIANT};
     const double bytes = 2.0 * A.vh * (2 * half_field_bytes(1, prec) + 4 * link_block_bytes(1, link_prec(prec), recon));
